@@ -117,7 +117,7 @@ def draw(rng):
     if kind == "host":
         return c
     cv = rng.choice(["none", "none", "table"] + (["network"] if coef in ("manufactured", "e1")
-                                                 and n * steps * N < 2e9 else []))
+                                                 and n * steps * N < 4e8 else []))
     c.update(cv=cv, ragged=rng.random() < 0.3, knot_steps=rng.random() < 0.2)
     if kind == "calibrate":
         return c
