@@ -321,8 +321,8 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
                                 void* cuda_stream);
 
 /* FP64 BiCGSTAB for G u = b (Eq. 23), all on the device; u (device double[n])
- * is overwritten (initial guess 0).  Synchronizes the stream to read the
- * residual every few iterations.  Returns ENOCONV if ||b - G u|| > rtol ||b||
+ * is overwritten (initial guess 0).  One cooperative kernel launch; synchronizes the
+ * stream to read the outcome.  Returns ENOCONV if ||b - G u|| > rtol ||b||
  * after maxit iterations; *iters (nullable) gets the iteration count. */
 pdds_status pdds_solve(pdds_ctx* ctx, const pdds_csr* G, const double* b, double* u,
                        double rtol, int32_t maxit, int32_t* iters, void* cuda_stream);
@@ -455,12 +455,12 @@ pdds_status pdds_set_control_variate_grid(pdds_ctx* ctx, const float* grad_xy, i
  * accounting or fail, and latency-critical code that cannot accept the implicit
  * synchronization of cudaMalloc/cudaFree.  It needs no context and calls no
  * cudaMalloc, cudaFree or allocating library routine: its scratch (six work
- * vectors and the recurrence scalars) is a static device array of
- * 6 * 131072 + 32 doubles (6.3 MB) that every GPU loading this library holds
+ * vectors, the recurrence scalars and the partial sums) is a static device array of
+ * 6 * 131072 + 4096 doubles (6.3 MB) that every GPU loading this library holds
  * until the process exits.
  *   G, b, u, rtol, maxit, iters, cuda_stream: as for pdds_solve (all device
- *     pointers; u is overwritten, initial guess 0; the stream is synchronized
- *     every few iterations to read the residual).
+ *     pointers; u is overwritten, initial guess 0; the stream is synchronized to
+ *     read the outcome).
  *   G->n must be in [1, 131072]; larger systems are rejected with PDDS_EINVAL
  *     before any device work (use pdds_solve).
  * The first call on each device looks up the array's device address with that

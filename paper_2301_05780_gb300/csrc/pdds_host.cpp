@@ -561,6 +561,27 @@ pdds_status assemble_impl(pdds_ctx* c, const int64_t* N, int64_t Nu, double dt, 
   return PDDS_OK;
 }
 
+// A solve of G u = b with the context's scratch (allocated once).
+pdds_status solve_job(pdds_ctx* c, const pdds_csr& G, const double* b, double* u,
+                      pdds::SolveJob& J) {
+  if (!c->d_work) CK(c, dalloc(&c->d_work, pdds::bicgstab_work_doubles(c->geo.n)));
+  if (!c->d_scalars)
+    CK(c, cudaMalloc(reinterpret_cast<void**>(&c->d_scalars), pdds::bicgstab_scalars_bytes()));
+  J = pdds::SolveJob{G.row_ptr, G.col, G.val, b, u, c->geo.n, c->geo.nnz, c->d_work, c->d_scalars,
+                     0, 0.0, 0};
+  return PDDS_OK;
+}
+// Records a finished solve in the context's counters.
+pdds_status solve_status(pdds_ctx* c, const pdds::SolveJob& J) {
+  c->st.solve_iters = J.iters;
+  c->st.solve_relres = J.relres;
+  if (J.converged == 1) return PDDS_OK;
+  char buf[200];
+  std::snprintf(buf, sizeof buf, "solve: no convergence after %d iterations (relres %.3e)%s",
+                J.iters, J.relres, pdds::bicgstab_stop_reason(J.converged));
+  return fail(c, PDDS_ENOCONV, buf);
+}
+
 }  // namespace
 
 namespace pdds {
@@ -1230,27 +1251,13 @@ pdds_status pdds_solve(pdds_ctx* c, const pdds_csr* G, const double* b, double* 
     return fail(c, PDDS_EINVAL, "solve: G sized differently from pdds_num_knots");
   if (!(rtol > 0) || maxit < 1) return fail(c, PDDS_EINVAL, "solve: need rtol > 0, maxit >= 1");
   (void)cudaGetLastError();
-  const int64_t n = c->geo.n;
-  if (!c->d_work) {
-    CK(c, dalloc(&c->d_work, pdds::bicgstab_work_doubles(n)));
-    CK(c, cudaMalloc(reinterpret_cast<void**>(&c->d_scalars), pdds::bicgstab_scalars_bytes()));
-  }
-  int32_t it = 0;
-  double rel = 0;
-  int conv = 0, nl = 0;
-  CK(c, pdds::bicgstab_device(G->row_ptr, G->col, G->val, b, u, n, c->d_work, c->d_scalars, rtol,
-                              maxit, &it, &rel, &conv, &nl, (cudaStream_t)stream));
-  c->st.solve_iters = it;
-  c->st.solve_relres = rel;
+  pdds::SolveJob J;
+  if (pdds_status e = solve_job(c, *G, b, u, J)) return e;
+  int nl = 0;
+  CK(c, pdds::bicgstab_batch(&J, 1, rtol, maxit, &nl, (cudaStream_t)stream));
   c->st.kernel_launches += nl;
-  if (iters) *iters = it;
-  if (conv != 1) {
-    char buf[200];
-    std::snprintf(buf, sizeof buf, "solve: no convergence after %d iterations (relres %.3e)%s",
-                  it, rel, pdds::bicgstab_stop_reason(conv));
-    return fail(c, PDDS_ENOCONV, buf);
-  }
-  return PDDS_OK;
+  if (iters) *iters = J.iters;
+  return solve_status(c, J);
 }
 
 pdds_status pdds_assemble_solve_host(pdds_ctx* c, const int64_t* N_host, int64_t Nu, double dt,
@@ -1469,6 +1476,8 @@ pdds_status pdds_assemble_solve_batch_host(pdds_ctx* const* ctxs, int32_t count,
       if (Nh[k] < 0 || Nh[k] > 0x7fffffffll)
         return fail(c0, PDDS_EINVAL, "assemble_solve_batch_host: every N_k must be in [0, 2^31)");
   }
+  if (!(rtol > 0) || maxit < 1)
+    return fail(c0, PDDS_EINVAL, "assemble_solve_batch_host: need rtol > 0, maxit >= 1");
   cudaStream_t s = (cudaStream_t)stream;
   // Device buffers: each context's own end-to-end scratch (kept for reuse).
   std::vector<pdds_csr> Gs(count);
@@ -1497,16 +1506,17 @@ pdds_status pdds_assemble_solve_batch_host(pdds_ctx* const* ctxs, int32_t count,
   if (pdds_status e = pdds_assemble_batch(ctxs, count, N_host ? Nd.data() : nullptr, Nu, dt, seed,
                                           Gp.data(), bd.data(), stream))
     return e;
+  // The solves of all problems side by side in one launch, each on its own CTAs.
   pdds_status worst = PDDS_OK;
-  int launches = c0->st.kernel_launches;
-  for (int i = 0; i < count; ++i) {
-    pdds_ctx* c = ctxs[i];
-    const int before = c->st.kernel_launches;
-    pdds_status se = pdds_solve(c, &Gs[i], c->e_b, c->e_u, rtol, maxit, nullptr, stream);
-    if (se != PDDS_OK && se != PDDS_ENOCONV) return c == c0 ? se : fail(c0, se, c->err);
-    if (se == PDDS_ENOCONV) worst = PDDS_ENOCONV;
-    launches += c->st.kernel_launches - before;
-  }
+  std::vector<pdds::SolveJob> jobs(count);
+  for (int i = 0; i < count; ++i)
+    if (pdds_status e = solve_job(ctxs[i], Gs[i], ctxs[i]->e_b, ctxs[i]->e_u, jobs[i]))
+      return ctxs[i] == c0 ? e : fail(c0, e, ctxs[i]->err);
+  int nl = 0;
+  CK(c0, pdds::bicgstab_batch(jobs.data(), count, rtol, maxit, &nl, s));
+  const int launches = c0->st.kernel_launches + nl;
+  for (int i = 0; i < count; ++i)
+    if (solve_status(ctxs[i], jobs[i]) == PDDS_ENOCONV) worst = PDDS_ENOCONV;
   for (int i = 0; i < count; ++i) {
     pdds_ctx* c = ctxs[i];
     const int64_t n = c->geo.n, nnz = c->geo.nnz;

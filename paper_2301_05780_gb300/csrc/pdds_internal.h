@@ -179,8 +179,24 @@ cudaError_t launch_boundary_samples(int coef, const double dom[4], const double 
 
 // FP64 BiCGSTAB building blocks (pdds_solve.cu).
 struct SolveScalars;
+struct SolveJob {           // one problem of a batched solve
+  const int32_t* rp;
+  const int32_t* ci;
+  const double* val;
+  const double* b;
+  double* x;
+  int64_t n, nnz;
+  double* work;             // bicgstab_work_doubles(n)
+  SolveScalars* sc;         // bicgstab_scalars_bytes()
+  int32_t iters;            // out: iterations, ||b - A x|| / ||b||, and 1 (converged),
+  double relres;            //   0 (maxit) or a negative breakdown code
+  int converged;
+};
+// Solves every job (device pointers); synchronizes the stream.
+cudaError_t bicgstab_batch(SolveJob* jobs, int count, double rtol, int32_t maxit, int* launches,
+                           cudaStream_t stream);
 cudaError_t bicgstab_device(const int32_t* row_ptr, const int32_t* col, const double* val,
-                            const double* b, double* x, int64_t n, double* work,
+                            const double* b, double* x, int64_t n, int64_t nnz, double* work,
                             SolveScalars* sc, double rtol, int32_t maxit, int32_t* iters,
                             double* relres, int* converged, int* launches, cudaStream_t stream);
 size_t bicgstab_work_doubles(int64_t n);
