@@ -569,52 +569,158 @@ __device__ __forceinline__ bool outside_box(float X, float Y, float bx0, float b
   return (X > bx1) | (X < bx0) | (Y > by1) | (Y < by0);
 }
 
-template <bool B>
-struct BoolTag {
-  static constexpr bool value = B;
-};
-
 template <int COEF>
 __host__ __device__ constexpr bool uses_angles() {  // the coefficients take sines of the position
   return COEF == PDDS_COEF_MANUFACTURED || COEF == PDDS_COEF_VARSIGMA ||
          COEF == PDDS_COEF_POISSON_E1;
 }
 
-// P.calls_per_check Philox calls (two steps each) of one lane's path on the
-// naive exit, between two exit checks of the warp: the two steps of a call are
-// taken without a branch between them -- the second one starts from the first
-// one's result and is dropped when the first one left the patch or reached
-// the step cap.  DIRECT: the coefficient sines take the angle without
-// reduction (the launch's domains allow it), a compile-time choice so that the
-// step carries no branch on it.
-template <int COEF, int CV, bool DIRECT>
-__device__ __forceinline__ void step_calls(const Stage& H, const float* tile,
-                                               const KParams& P, uint32_t p, uint32_t kk,
-                                               uint32_t tagw, float xk, float yk, float h,
-                                               float hl2, float sqh, int kmax, float bx0,
-                                               float bx1, float by0, float by1, int& n, float& X,
-                                               float& Y, float& Sx, float& Z, float& XI,
-                                               bool& exited, bool& trunc) {
+// The exit test after a step: outside the lane's box (moved inwards by the
+// largest Gobet-Menozzi shift in the extended kernels), and, where s varies,
+// beyond a side moved by its own shift.
+template <int COEF, bool EXT>
+__device__ __forceinline__ bool left_patch(const Stage& H, const float* tile, float xk, float yk,
+                                           float X, float Y, float bx0, float bx1, float by0,
+                                           float by1, float gmc, bool direct) {
+  bool out = outside_box(X, Y, bx0, bx1, by0, by1);
+  if constexpr (EXT && !const_sigma<COEF>()) {
+    if (out && gmc > 0.f) out = gm_outside<COEF>(H, tile, tile, xk, yk, X, Y, gmc, direct);
+  }
+  return out;
+}
+
+// What one lane's path carries from step to step, and what stays fixed.
+struct PathState {
+  float X, Y, S, Z, XI;
+  int n;
+  bool exited;
+};
+struct PathConst {
+  const Stage* H;
+  const float* tile;
+  uint32_t p, kk, tagw;
+  float xk, yk, h, hl2, sqh, bx0, bx1, by0, by1, gmc;
+};
+
+// The two steps of one Philox call, from the normals gA and gB, without a
+// branch between them; the second one is dropped when the first one left the
+// patch.  The caller has made sure that the step cap is not reached.
+template <int COEF, int CV, bool EXT, bool DIRECT>
+__device__ __forceinline__ void step_pair(const PathConst& c, const KParams& P, float2 gA, float2 gB,
+                                          PathState& s) {
+  float X1 = s.X, Y1 = s.Y, S1 = s.S, Z1 = s.Z, XI1 = s.XI;
+  em_step<COEF, CV>(*c.H, c.tile, P, DIRECT, c.xk, c.yk, c.h, c.hl2, c.sqh, gA, X1, Y1, S1, Z1, XI1);
+  const bool e1 = left_patch<COEF, EXT>(*c.H, c.tile, c.xk, c.yk, X1, Y1, c.bx0, c.bx1, c.by0, c.by1,
+                                        c.gmc, DIRECT);
+  s.X = X1; s.Y = Y1; s.S = S1; s.Z = Z1; s.XI = XI1;
+  em_step<COEF, CV>(*c.H, c.tile, P, DIRECT, c.xk, c.yk, c.h, c.hl2, c.sqh, gB, s.X, s.Y, s.S, s.Z,
+                    s.XI);
+  const bool e2 = left_patch<COEF, EXT>(*c.H, c.tile, c.xk, c.yk, s.X, s.Y, c.bx0, c.bx1, c.by0,
+                                        c.by1, c.gmc, DIRECT);
+  s.n += 2;
+  s.exited = e1 | e2;
+  if (e1) {
+    s.X = X1; s.Y = Y1; s.S = S1; s.Z = Z1; s.XI = XI1;
+    s.n -= 1;
+  }
+}
+
+// P.calls_per_check Philox calls (two steps each) of one lane's path between
+// two exit checks of the warp.  DIRECT: the coefficient sines take the angle
+// without reduction (the launch's domains allow it), a compile-time choice so
+// that the step carries no branch on it.
+// The step cap is tested once per visit: while it is out of reach of the whole
+// visit the loop carries no compare on n, and what the first step of a call
+// left behind is selected only when the path has exited, not in every call
+// (one GB300, against selects and cap compares in every call: manufactured set
+// 48.5 -> 46.9 ms at 1.4e10 path-steps, variable sigma 466 -> 461 ms at
+// 1.5e11, the paper's GM warm-up, until then one branch per step, 20.1 -> 18.9
+// ms at 4.4e9, its production run 46.9 -> 45.3 ms).
+template <int COEF, int CV, bool EXT, bool DIRECT>
+__device__ __forceinline__ void step_calls(const PathConst& c, const KParams& P, const PhiloxPath& ph,
+                                           int kmax, PathState& s, bool& trunc) {
+  constexpr bool kPre = EXT && CV == 0;
+  // (the tabulated set's extended kernel spills more with two exact exit tests
+  // per call: 2 % slower, so it goes step by step)
+  constexpr bool kPair = !(EXT && COEF == PDDS_COEF_TABLE);
+  if (kPair && !(s.n & 1) && s.n + 2 * P.calls_per_check < kmax) {
 #pragma unroll 1
-  for (int pair = 0; pair < P.calls_per_check && !exited; ++pair) {
-    const uint4 r = philox4x32_10(make_uint4((uint32_t)(n >> 1), p, kk, tagw), P.round_keys);
+    for (int call = P.calls_per_check; call > 0 && !s.exited; --call) {
+      const uint4 r = kPre ? philox_step((uint32_t)(s.n >> 1), ph, P.round_keys)
+                           : philox4x32_10(make_uint4((uint32_t)(s.n >> 1), c.p, c.kk, c.tagw),
+                                           P.round_keys);
+      float2 gA, gB;
+      box_muller4(r, gA, gB);
+      step_pair<COEF, CV, EXT, DIRECT>(c, P, gA, gB, s);
+    }
+  } else {
+    // step by step: near the step cap, or resuming a mixed run at an odd step
+#pragma unroll 1
+    for (int call = P.calls_per_check; call > 0 && !s.exited; --call) {
+      const uint4 r = kPre && !kPair ? philox_step((uint32_t)(s.n >> 1), ph, P.round_keys)
+                                     : philox4x32_10(make_uint4((uint32_t)(s.n >> 1), c.p, c.kk, c.tagw),
+                                                     P.round_keys);
+      float2 gA, gB;
+      box_muller4(r, gA, gB);
+      auto step = [&](float2 g) {
+        em_step<COEF, CV>(*c.H, c.tile, P, DIRECT, c.xk, c.yk, c.h, c.hl2, c.sqh, g, s.X, s.Y, s.S, s.Z,
+                          s.XI);
+        ++s.n;
+        s.exited = left_patch<COEF, EXT>(*c.H, c.tile, c.xk, c.yk, s.X, s.Y, c.bx0, c.bx1, c.by0,
+                                         c.by1, c.gmc, DIRECT);
+        if (!s.exited && s.n >= kmax) { s.exited = true; trunc = true; }
+      };
+      // a call serves steps 2q and 2q + 1; a path that resumes at an odd step
+      // takes the second half of its call
+      if constexpr (kPair) {
+#pragma unroll 1
+        for (int half = s.n & 1; half < 2 && !s.exited; ++half) step(half ? gB : gA);
+      } else {
+        if (!(s.n & 1)) step(gA);
+        if (!s.exited) step(gB);
+      }
+    }
+  }
+}
+
+// Few paths left in a warp (nothing more to hand out, or a problem smaller
+// than the chip): a path's normals depend on its counter alone, so the idle
+// lanes take Philox calls ahead for the stepping ones.  `stepping`: the m <= 16
+// lanes that step.  Lane l takes call l % G (G = 32 / m, a power of two) of the
+// path with rank l / G, and the owner of that path fetches the G calls' normals
+// by shuffles, one call (two steps) at a time.  A lone path thus waits for one
+// Philox call and Box-Muller (about 300 cycles of latency) per 64 steps instead
+// of per two (2.9e5 Laplace paths 0.76 -> 0.63 ms in units of 128, 1.2e6
+// variable-sigma paths 5.6 -> 5.1 ms).  Same counters, same arithmetic: the paths are the same bit for
+// bit.  The caller has made sure that no path reaches its cap in 2 G `rounds` steps.
+template <int COEF, int CV, bool EXT, bool DIRECT>
+__device__ __forceinline__ void coop_calls(const PathConst& c, const KParams& P, unsigned stepping,
+                                           int log2g, int rounds, PathState& s) {
+  const int lane = threadIdx.x & 31;
+  const bool mine = (stepping >> lane) & 1;
+  // the lane whose path has rank lane / G: the bit of that rank in `stepping`
+  const int rank = lane >> log2g;
+  int owner = 0;
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1)
+    if (__popc(stepping & ((1u << (owner + w)) - 1u)) <= rank) owner += w;
+  if (rank >= __popc(stepping)) owner = lane;
+  const uint32_t p = __shfl_sync(kFull, c.p, owner), kk = __shfl_sync(kFull, c.kk, owner),
+                 tagw = __shfl_sync(kFull, c.tagw, owner);
+  const uint32_t ahead = (uint32_t)(lane & ((1 << log2g) - 1));
+  // this lane's path is served by lanes src .. src + G - 1
+  const int src = __popc(stepping & ((1u << lane) - 1u)) << log2g;
+  for (int r = 0; r < rounds; ++r) {
+    const uint32_t q = (uint32_t)__shfl_sync(kFull, s.n >> 1, owner) + ahead;
     float2 gA, gB;
-    box_muller4(r, gA, gB);
-    float X1 = X, Y1 = Y, S1 = Sx, Z1 = Z, XI1 = XI;
-    em_step<COEF, CV>(H, tile, P, DIRECT, xk, yk, h, hl2, sqh, gA, X1, Y1, S1, Z1, XI1);
-    const bool e1 = outside_box(X1, Y1, bx0, bx1, by0, by1);
-    float X2 = X1, Y2 = Y1, S2 = S1, Z2 = Z1, XI2 = XI1;
-    em_step<COEF, CV>(H, tile, P, DIRECT, xk, yk, h, hl2, sqh, gB, X2, Y2, S2, Z2, XI2);
-    const bool e2 = outside_box(X2, Y2, bx0, bx1, by0, by1);
-    const bool first = e1 || (n + 1 >= kmax);
-    X = first ? X1 : X2;
-    Y = first ? Y1 : Y2;
-    Sx = first ? S1 : S2;
-    Z = first ? Z1 : Z2;
-    if constexpr (CV == 2) XI = first ? XI1 : XI2;
-    n += first ? 1 : 2;
-    exited = first ? e1 : e2;
-    if (!exited && n >= kmax) { exited = true; trunc = true; }
+    box_muller4(philox4x32_10(make_uint4(q, p, kk, tagw), P.round_keys), gA, gB);
+#pragma unroll 1
+    for (int j = 0; j < (1 << log2g); ++j) {
+      const int from = (src + j) & 31;
+      const float2 a = f2(__shfl_sync(kFull, gA.x, from), __shfl_sync(kFull, gA.y, from));
+      const float2 b = f2(__shfl_sync(kFull, gB.x, from), __shfl_sync(kFull, gB.y, from));
+      if (mine && !s.exited) step_pair<COEF, CV, EXT, DIRECT>(c, P, a, b, s);
+    }
   }
 }
 
@@ -1138,79 +1244,28 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
             if (!exited && n >= kmax) { exited = true; trunc = true; }
           }
         }
-      } else if (!EXT && alive && !exited) {
+      } else {
         const Stage& H = S.st(st);
-        const float* tile = S.tile(st, 0);
-        if (uses_angles<COEF>() && P.trig_direct)
-          step_calls<COEF, CV, uses_angles<COEF>()>(H, tile, P, p, kk, tagw, xk, yk, h, hl2,
-                                                        sqh, kmax, bx0, bx1, by0, by1, n, X, Y,
-                                                        Sx, Z, XI, exited, trunc);
-        else
-          step_calls<COEF, CV, false>(H, tile, P, p, kk, tagw, xk, yk, h, hl2, sqh, kmax,
-                                          bx0, bx1, by0, by1, n, X, Y, Sx, Z, XI, exited, trunc);
-      } else if (alive && !exited) {
-       // extended-exit kernels (per-knot steps, Gobet-Menozzi exits, the mixed
-       // GM/EM run): P.calls_per_check Philox calls between exit checks, one
-       // branch per step (the two-step form spills more here)
-       // (the angle-reduction choice is a template constant here too)
-       auto ext_calls = [&](auto direct_tag) {
-        constexpr bool kDirect = decltype(direct_tag)::value;
-#pragma unroll 1
-         for (int pair = 0; pair < P.calls_per_check; ++pair) {
-          if (exited) break;
-          const uint4 r = kPhiloxPre ? philox_step((uint32_t)(n >> 1), ph, P.round_keys)
-                            : philox4x32_10(make_uint4((uint32_t)(n >> 1), p, kk, tagw), P.round_keys);
-          float z[4];
-          box_muller(r.x, r.y, z[0], z[1]);
-          box_muller(r.z, r.w, z[2], z[3]);
-#pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            // a Philox call serves steps 2q and 2q + 1; a mixed-run path that
-            // resumes at an odd step takes the second half of its call
-            if (!exited && (!kMixed || half >= (n & 1))) {
-              const Stage& H = S.st(st);
-              float s, ddx, ddy, c, f;
-              coeffs<COEF>(H, S.tile(st, 0), S.tile(st, 1), xk + X, yk + Y, X, Y, kDirect,
-                           s, ddx, ddy, c, f);
-              float Yw = 1.0f;
-              if constexpr (has_c<COEF>()) {
-                Yw = ex2_approx(Sx);
-                Z = fmaf(-f * Yw, h, Z);  // dZ = -f Y dt
-                Sx = fmaf(c, hl2, Sx);    // dY = c Y dt, Y = 2^S with S = log2(e) int c dt
-              } else if constexpr (has_f<COEF>()) {
-                Z = fmaf(-f, h, Z);       // c = 0: Y = 1
-              }
-              // dX = d dt + s dW with dW = sqrt(h) z: s sqrt(h) once, then two FMAs
-              const float ssh = s * sqh;
-              if constexpr (CV == 2) {
-                // dxi = -Y s grad u0 . dW with grad u0 from the table (Eq. 37, Sec. 4.2)
-                float gx, gy;
-                // a control variate never runs batched (pdds_assemble_batch refuses
-                // it), so the table is problem 0's, read from the launch constants:
-                // no per-step loads of the problem descriptor
-                cv_table_grad(P.prob0, xk + X, yk + Y, gx, gy);
-                XI = fmaf(-Yw * ssh, fmaf(gx, z[2 * half], gy * z[2 * half + 1]), XI);
-              }
-              if constexpr (has_drift<COEF>()) {
-                X = fmaf(ssh, z[2 * half], fmaf(ddx, h, X));
-                Y = fmaf(ssh, z[2 * half + 1], fmaf(ddy, h, Y));
-              } else {
-                X = fmaf(ssh, z[2 * half], X);
-                Y = fmaf(ssh, z[2 * half + 1], Y);
-              }
-              ++n;
-              exited = (X > bx1) | (X < bx0) | (Y > by1) | (Y < by0);
-              if constexpr (EXT && !const_sigma<COEF>()) {
-                if (exited && gmc > 0.f) exited = gm_outside<COEF>(H, S.tile(st, 0), S.tile(st, 1),
-                                                                xk, yk, X, Y, gmc, kDirect);
-              }
-              if (!exited && n >= kmax) { exited = true; trunc = true; }
-            }
-          }
-         }
-       };
-       if (uses_angles<COEF>() && P.trig_direct) ext_calls(BoolTag<uses_angles<COEF>()>{});
-       else ext_calls(BoolTag<false>{});
+        const PathConst c{&H, S.tile(st, 0), p, kk, tagw, xk, yk, h, hl2, sqh, bx0, bx1, by0, by1, gmc};
+        PathState s{X, Y, Sx, Z, XI, n, exited};
+        const unsigned todo = __ballot_sync(kFull, alive && !exited);
+        // direct: the sines take their angles without reduction (all launches
+        // on the domains of the paper's problem and the benchmarks)
+        constexpr bool kAngles = uses_angles<COEF>();
+        const int m = __popc(todo), log2g = m > 1 ? __clz(m - 1) - 27 : 5;  // 32 / m paths, rounded down
+        const int rounds = max(1, P.calls_per_check >> log2g);
+        // (not for the tabulated set: its steps wait for shared-memory lookups,
+        // not for Philox, and ran 6 % slower this way)
+        if (COEF != PDDS_COEF_TABLE && log2g > 0 && todo != 0 &&
+            __all_sync(kFull, !((todo >> lane) & 1) ||
+                                  (!(n & 1) && n + ((2 * rounds) << log2g) < kmax))) {
+          if (kAngles && P.trig_direct) coop_calls<COEF, CV, EXT, kAngles>(c, P, todo, log2g, rounds, s);
+          else coop_calls<COEF, CV, EXT, false>(c, P, todo, log2g, rounds, s);
+        } else if (alive && !exited) {
+          if (kAngles && P.trig_direct) step_calls<COEF, CV, EXT, kAngles>(c, P, ph, kmax, s, trunc);
+          else step_calls<COEF, CV, EXT, false>(c, P, ph, kmax, s, trunc);
+        }
+        X = s.X; Y = s.Y; Sx = s.S; Z = s.Z; XI = s.XI; n = s.n; exited = s.exited;
       }
       const unsigned ex = __ballot_sync(kFull, alive && exited);
       const unsigned stepping = __ballot_sync(kFull, alive && !exited);
