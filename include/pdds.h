@@ -156,7 +156,10 @@ pdds_status pdds_set_step_cap(pdds_ctx* ctx, int64_t k_max);
 /* Launch shape of the path kernel: threads per CTA (multiple of 32, <= 1024),
  * CTAs per SM (0 = occupancy maximum), paths per work unit (>= 32) and the
  * number of exited lanes a warp gathers before resolving exits (1..32).
- * Zeros keep the current value.  pdds_autotune picks them by measurement. */
+ * Zeros keep the current value.  pdds_autotune picks them by measurement.  A
+ * field that neither has set is the library's choice, launch by launch, from
+ * the problem's paths, steps per path and shared memory; pdds_get_launch then
+ * reports 256 / 0 / 4096 / 4. */
 pdds_status pdds_set_launch(pdds_ctx* ctx, int32_t block, int32_t ctas_per_sm,
                             int32_t unit_paths, int32_t exit_batch);
 pdds_status pdds_get_launch(const pdds_ctx* ctx, int32_t* block, int32_t* ctas_per_sm,

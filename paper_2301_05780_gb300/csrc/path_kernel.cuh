@@ -916,18 +916,20 @@ __device__ bool load_unit(const Smem& S, int s, int q, const KParams& P, int64_t
     const ProbDesc& D = prob_desc(P, prob);
     const int64_t uu = (int64_t)u - P.prob_unit_prefix[prob];
     int64_t j;
-    int64_t Nk;
+    int64_t Nk, size;
     if (D.knot_unit_prefix == nullptr) {
       k = (int)(uu / D.units_per_knot);
       j = uu - (int64_t)k * D.units_per_knot;
       Nk = D.n_paths;
+      size = D.unit_paths;
     } else {
       k = (int)upper_bound_i64(D.knot_unit_prefix, (int64_t)D.n + 1, uu) - 1;
       j = uu - D.knot_unit_prefix[k];
       Nk = D.n_per_knot[k];
+      size = D.knot_unit_prefix[D.n + 1];
     }
-    pb = j * P.unit_paths;
-    pe = min(Nk, pb + P.unit_paths);
+    pb = j * size;
+    pe = min(Nk, pb + size);
   }
   prob = __shfl_sync(kFull, prob, 0);
   k = __shfl_sync(kFull, k, 0);

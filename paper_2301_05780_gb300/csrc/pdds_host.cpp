@@ -230,8 +230,11 @@ struct pdds_ctx {
   int64_t* d_path_prefix = nullptr;
   int64_t* d_prob_prefix = nullptr;
   // launch configuration
+  // launch shape of pdds_set_launch / pdds_autotune; a field that neither has
+  // set is the library's choice per launch (plan_launch)
   int block = 256, ctas_per_sm = 0, exit_batch = 4;
   int64_t unit_paths = 4096;
+  bool auto_block = true, auto_unit = true, auto_batch = true;
   int64_t k_max = 0;
   uint32_t tag = 0;  // Philox tag (fourth counter word) of single-problem calls
   int net_engine = PDDS_NET_TCGEN05;  // tensor-core engine of the in-path network
@@ -424,10 +427,69 @@ int64_t default_kmax(const pdds_ctx* c, double dt) {
   return (int64_t)std::ceil(40.0 * T / dt);
 }
 
+// The shape of one path-kernel launch.
+struct LaunchPlan {
+  int cv = 0, block = 0, grid = 0, exit_batch = 0;
+  size_t smem = 0;
+  int64_t unit_paths = 0;  // 0: auto_unit_paths
+  int64_t warps() const { return block / 32; }
+};
+
+// Fields that pdds_set_launch or pdds_autotune have set are kept; the others:
+//  - block: the smallest, up to 256 threads, that keeps 24 warps resident per
+//    SM (or as many as any): small CTAs contend less on their two staged units
+//    (paths of 11 steps: 10.2 ms with 64 threads, 38.7 with 256; long paths
+//    within 1 %); where shared memory limits the CTAs (coefficient tiles, wide
+//    stencils) more warps have to share one (tabulated fields, three CTAs per
+//    SM: 31 ms with 192 or 256 threads, 57 with 64, 38 with 384);
+//  - exit batch: 4 lanes, 8 where a path takes fewer steps than two visits of
+//    the step loop (2 % on paths of 11 steps, 2-4 % slower on long ones).
+pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob, size_t sbytes,
+                        double dt, LaunchPlan& L) {
+  // cv 3: the in-path network on tcgen05 (the warpgroup kernel)
+  L.cv = nprob == 1 ? c->cv_mode : 0;
+  if (L.cv == 1 && c->net_engine == PDDS_NET_TCGEN05) L.cv = 3;
+  // network kernels keep the staged network at the start of dynamic shared
+  // memory (the tcgen05 kernel: its swizzled operand tiles)
+  L.smem = 2 * sbytes + (L.cv == 1   ? round_up(pdds::mlp_image_bytes(), 128)
+                         : L.cv == 3 ? pdds::net_smem_bytes()
+                                     : 0);
+  CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, L.smem));
+  int per_sm = 0;
+  if (L.cv == 3) {
+    L.block = 128;  // one warpgroup
+  } else if (!c->auto_block || c->ctas_per_sm > 0) {
+    L.block = L.cv == 1 ? std::min(c->block, 256) : c->block;
+  } else {
+    static const int blocks[] = {64, 128, 192, 256};
+    int warps[4] = {0}, most = 0;
+    for (int i = 0; i < 4; ++i) {
+      int ctas = 0;
+      CK(c, pdds::path_kernel_occupancy(coef_id, rec, L.cv, ext, blocks[i], L.smem, &ctas));
+      warps[i] = ctas * blocks[i] / 32;
+      most = std::max(most, warps[i]);
+    }
+    for (int i = 3; i >= 0; --i)
+      if (warps[i] >= std::min(most, 24)) L.block = blocks[i];
+  }
+  per_sm = c->ctas_per_sm;
+  if (per_sm <= 0) {
+    CK(c, pdds::path_kernel_occupancy(coef_id, rec, L.cv, ext, L.block, L.smem, &per_sm));
+    if (per_sm <= 0) return fail(c, PDDS_EINVAL, "launch: block/shared memory too large");
+  }
+  // tcgen05 kernel: 96 TMEM columns per CTA, 512 per SM
+  if (L.cv == 3) per_sm = std::min(per_sm, 512 / 96);
+  L.grid = c->num_sms * per_sm;
+  // (the warpgroup kernel steps 128 paths at a time, however few are left)
+  L.unit_paths = c->auto_unit && L.cv != 3 ? 0 : c->unit_paths;
+  L.exit_batch = !c->auto_batch ? c->exit_batch : mean_steps_estimate(c, dt) < 32.0 ? 8 : 4;
+  return PDDS_OK;
+}
+
 // Everything one or more problems need for one persistent launch.
 // ext: extended-exit kernel (per-knot steps and/or the Gobet-Menozzi shift gm).
-pdds_status run_paths(pdds_ctx* c, const ProbDesc& p0, const ProbDesc* d_probs, int nprob,
-                      double dt, uint64_t seed, int64_t kmax, pdds::PathRecordDev* rec,
+pdds_status run_paths(pdds_ctx* c, const LaunchPlan& L, const ProbDesc& p0, const ProbDesc* d_probs,
+                      int nprob, double dt, uint64_t seed, int64_t kmax, pdds::PathRecordDev* rec,
                       cudaStream_t stream, size_t sbytes, int max_slots, int tile_w, int tile_h,
                       int coef_id, bool ext = false, bool gm = false,
                       pdds::PathRecordDev* rec_gm = nullptr) {
@@ -436,9 +498,8 @@ pdds_status run_paths(pdds_ctx* c, const ProbDesc& p0, const ProbDesc* d_probs, 
   kp.probs = d_probs;
   kp.nprob = nprob;
   kp.prob_unit_prefix = c->d_prob_prefix;
-  kp.exit_batch = c->exit_batch;
+  kp.exit_batch = L.exit_batch;
   kp.calls_per_check = c->batch_calls > 0 ? c->batch_calls : calls_per_check(c, dt);
-  kp.unit_paths = c->unit_paths;
   kp.scratch = c->d_scratch;
   kp.records = rec;
   kp.key0 = (uint32_t)seed;
@@ -463,9 +524,7 @@ pdds_status run_paths(pdds_ctx* c, const ProbDesc& p0, const ProbDesc* d_probs, 
   const double kmax_eff = ext && c->d_hknot && c->h_min < dt ? (double)kmax * dt / c->h_min
                                                              : (double)kmax;
   kp.wait_ns = c->wait_s > 0 ? (uint64_t)(c->wait_s * 1e9) : (uint64_t)(10e9 + 4000.0 * kmax_eff);
-  // cv 3: the in-path network on tcgen05 (the warpgroup kernel)
-  int cv = nprob == 1 ? c->cv_mode : 0;
-  if (cv == 1 && c->net_engine == PDDS_NET_TCGEN05) cv = 3;
+  const int cv = L.cv;
   kp.mlp = cv == 1 || cv == 3 ? c->d_mlp : nullptr;
   {
     // the largest |coordinate| of the launch's domains (problem 0 here, the
@@ -482,22 +541,8 @@ pdds_status run_paths(pdds_ctx* c, const ProbDesc& p0, const ProbDesc* d_probs, 
   }
   // the network step is ~10x heavier: wait bounds scale with it
   if ((cv == 1 || cv == 3) && c->wait_s <= 0) kp.wait_ns = (uint64_t)(10e9 + 40000.0 * kmax_eff);
-  // network kernels keep the staged network at the start of dynamic shared
-  // memory (the tcgen05 kernel: its swizzled operand tiles)
-  const size_t smem = 2 * sbytes + (cv == 1   ? round_up(pdds::mlp_image_bytes(), 128)
-                                    : cv == 3 ? pdds::net_smem_bytes()
-                                              : 0);
-  CK(c, pdds::set_path_kernel_smem(coef_id, rec != nullptr, cv, ext, smem));
-  // network: <= 256 threads; the tcgen05 kernel takes one warpgroup
-  const int block = cv == 1 ? std::min(c->block, 256) : cv == 3 ? 128 : c->block;
-  int per_sm = c->ctas_per_sm;
-  if (per_sm <= 0) {
-    CK(c, pdds::path_kernel_occupancy(coef_id, rec != nullptr, cv, ext, block, smem, &per_sm));
-    if (per_sm <= 0) return fail(c, PDDS_EINVAL, "launch: block/shared memory too large");
-  }
-  // tcgen05 kernel: 96 TMEM columns per CTA, 512 per SM
-  if (cv == 3) per_sm = std::min(per_sm, 512 / 96);
-  const int grid = c->num_sms * per_sm;
+  const int grid = L.grid, block = L.block;
+  const size_t smem = L.smem;
   c->st.path_grid = grid;
   c->st.path_block = block;
   if (c->timing) CK(c, cudaEventRecord(c->ev0, stream));
@@ -530,25 +575,29 @@ pdds_status assemble_impl(pdds_ctx* c, const int64_t* N, int64_t Nu, double dt, 
   CK(c, cudaMemsetAsync(G->val, 0, c->geo.nnz * 8, s));
   CK(c, cudaMemsetAsync(b, 0, c->geo.n * 8, s));
   CK(c, cudaMemsetAsync(c->d_scratch, 0, sizeof(pdds::Scratch), s));
+  const bool gm = (scheme < 0 ? c->scheme : scheme) == PDDS_SCHEME_GM;
+  const bool ext = gm || c->d_hknot != nullptr || c->interp == PDDS_INTERP_RBF;
+  LaunchPlan L;
+  if (pdds_status e = plan_launch(c, c->coef_id, rec != nullptr, ext, 1, stage_bytes(c), dt, L)) return e;
   ProbDesc D = make_prob(c, (int)c->tag);
   D.Gval = G->val;
   D.b = b;
   D.n_per_knot = N;
   D.n_paths = Nu;
   if (N) {
-    CK(c, pdds::launch_unit_prefix(N, c->geo.n, c->unit_paths, c->d_unit_prefix,
+    CK(c, pdds::launch_unit_prefix(N, c->geo.n, L.unit_paths, 1, L.grid, L.warps(), c->d_unit_prefix,
                                    c->d_path_prefix, &c->d_scratch->error, s));
     ++launches;
     D.knot_unit_prefix = c->d_unit_prefix;
     D.path_prefix = c->d_path_prefix;
   } else {
-    D.units_per_knot = ceil_div(Nu, c->unit_paths);
+    D.unit_paths = L.unit_paths ? L.unit_paths
+                                : pdds::auto_unit_paths(c->geo.n * Nu, L.grid, L.warps());
+    D.units_per_knot = ceil_div(Nu, D.unit_paths);
   }
   CK(c, pdds::launch_prob_prefix_single(D, c->d_prob_prefix, s));
   ++launches;
-  const bool gm = (scheme < 0 ? c->scheme : scheme) == PDDS_SCHEME_GM;
-  const bool ext = gm || c->d_hknot != nullptr || c->interp == PDDS_INTERP_RBF;
-  if (pdds_status e = run_paths(c, D, nullptr, 1, dt, seed, kmax,
+  if (pdds_status e = run_paths(c, L, D, nullptr, 1, dt, seed, kmax,
                                 reinterpret_cast<pdds::PathRecordDev*>(rec), s, stage_bytes(c),
                                 c->geo.max_slots, c->tile_w, c->tile_h, c->coef_id, ext, gm,
                                 reinterpret_cast<pdds::PathRecordDev*>(rec_gm)))
@@ -742,7 +791,7 @@ pdds_status pdds_create(const pdds_grid* grid, const pdds_coeffs* cf, pdds_ctx**
   if ((e = dalloc(&c->d_row_ptr, n + 1)) != cudaSuccess) return bail(e, "row_ptr alloc");
   if ((e = dalloc(&c->d_col, G.nnz)) != cudaSuccess) return bail(e, "col alloc");
   if ((e = dalloc(&c->d_scratch, 1)) != cudaSuccess) return bail(e, "scratch alloc");
-  if ((e = dalloc(&c->d_unit_prefix, n + 1)) != cudaSuccess) return bail(e, "prefix alloc");
+  if ((e = dalloc(&c->d_unit_prefix, n + 2)) != cudaSuccess) return bail(e, "prefix alloc");
   if ((e = dalloc(&c->d_path_prefix, n + 1)) != cudaSuccess) return bail(e, "prefix alloc");
   if ((e = dalloc(&c->d_prob_prefix, 2)) != cudaSuccess) return bail(e, "prefix alloc");
   if ((e = cudaMemcpy(c->d_knots, G.kd.data(), n * sizeof(KnotDesc), cudaMemcpyHostToDevice)) !=
@@ -815,10 +864,10 @@ pdds_status pdds_set_launch(pdds_ctx* c, int32_t block, int32_t per_sm, int32_t 
     return fail(c, PDDS_EINVAL, "set_launch: unit_paths in [32, 2^24]");
   if (exit_batch && (exit_batch < 1 || exit_batch > 32))
     return fail(c, PDDS_EINVAL, "set_launch: exit_batch in [1, 32]");
-  if (block) c->block = block;
+  if (block) { c->block = block; c->auto_block = false; }
   c->ctas_per_sm = per_sm;
-  if (unit_paths) c->unit_paths = unit_paths;
-  if (exit_batch) c->exit_batch = exit_batch;
+  if (unit_paths) { c->unit_paths = unit_paths; c->auto_unit = false; }
+  if (exit_batch) { c->exit_batch = exit_batch; c->auto_batch = false; }
   return PDDS_OK;
 }
 
@@ -895,6 +944,7 @@ pdds_status pdds_autotune(pdds_ctx* c, int64_t n_paths, double dt, uint64_t seed
       c->block = it->second.block;
       c->unit_paths = it->second.unit;
       c->exit_batch = it->second.batch;
+      c->auto_block = c->auto_unit = c->auto_batch = false;
       c->ctas_per_sm = 0;
       return PDDS_OK;
     }
@@ -934,6 +984,8 @@ pdds_status pdds_autotune(pdds_ctx* c, int64_t n_paths, double dt, uint64_t seed
   const int units[] = {256, 1024, 4096, 16384};
   const int batches[] = {2, 4, 8, 16};
   Shape best{c->block, (int)c->unit_paths, c->exit_batch};
+  const bool autos[3] = {c->auto_block, c->auto_unit, c->auto_batch};
+  c->auto_block = c->auto_unit = c->auto_batch = false;
   c->timing = true;
   c->ctas_per_sm = 0;
   std::vector<Shape> shapes;
@@ -981,7 +1033,12 @@ pdds_status pdds_autotune(pdds_ctx* c, int64_t n_paths, double dt, uint64_t seed
   c->unit_paths = best.unit;
   c->exit_batch = best.batch;
   cleanup();
-  if (st != PDDS_OK) return st;
+  if (st != PDDS_OK) {
+    c->auto_block = autos[0];
+    c->auto_unit = autos[1];
+    c->auto_batch = autos[2];
+    return st;
+  }
   std::lock_guard<std::mutex> lock(mu);
   cache[key] = best;
   return PDDS_OK;
@@ -1337,7 +1394,8 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
   // Graph key: everything the captured sequence depends on.
   std::vector<uint64_t> key = {(uint64_t)count, (uint64_t)Nu, (uint64_t)seed, (uint64_t)kmax,
                                (uint64_t)c0->block, (uint64_t)c0->ctas_per_sm,
-                               (uint64_t)c0->unit_paths, (uint64_t)c0->exit_batch};
+                               (uint64_t)c0->unit_paths, (uint64_t)c0->exit_batch,
+                               (uint64_t)(c0->auto_block + 2 * c0->auto_unit + 4 * c0->auto_batch)};
   uint64_t dtb;
   std::memcpy(&dtb, &dt, 8);
   key.push_back(dtb);
@@ -1351,6 +1409,14 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
   }
   if (!(c0->graph && key == c0->graph_key)) {
     if (c0->graph) { cudaGraphExecDestroy(c0->graph); c0->graph = nullptr; }
+    const size_t sb = [&] {
+      size_t x = pdds::stage_header_bytes() + round_up((size_t)max_slots * 8, 128);
+      if (c0->coef_id == PDDS_COEF_TABLE) x += round_up((size_t)2 * tw * th * 4, 128);
+      return round_up(x, 128);
+    }();
+    LaunchPlan L;
+    if (pdds_status e = plan_launch(c0, c0->coef_id, false, false, count == 1 ? 1 : 2, sb, dt, L))
+      return e;
     std::vector<ProbDesc> probs(count);
     for (int i = 0; i < count; ++i) {
       pdds_ctx* c = ctxs[i];
@@ -1363,7 +1429,10 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
         D.knot_unit_prefix = c->d_unit_prefix;
         D.path_prefix = c->d_path_prefix;
       } else {
-        D.units_per_knot = ceil_div(Nu, c0->unit_paths);
+        // the launch's paths are about `count` times this problem's
+        D.unit_paths = L.unit_paths ? L.unit_paths
+                                    : pdds::auto_unit_paths(count * c->geo.n * Nu, L.grid, L.warps());
+        D.units_per_knot = ceil_div(Nu, D.unit_paths);
       }
       probs[i] = D;
     }
@@ -1378,12 +1447,6 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
     }
     CK(c0, cudaStreamSynchronize(s));  // a previous replay may still read the old table
     CK(c0, cudaMemcpy(c0->d_batch, probs.data(), count * sizeof(ProbDesc), cudaMemcpyHostToDevice));
-    const size_t sb = [&] {
-      size_t x = pdds::stage_header_bytes() + round_up((size_t)max_slots * 8, 128);
-      if (c0->coef_id == PDDS_COEF_TABLE) x += round_up((size_t)2 * tw * th * 4, 128);
-      return round_up(x, 128);
-    }();
-    CK(c0, pdds::set_path_kernel_smem(c0->coef_id, false, 0, false, 2 * sb));
     // Capture on a private non-blocking stream (the legacy default stream
     // cannot be captured); the instantiated graph is launched on the caller's.
     if (!c0->cap_stream) CK(c0, cudaStreamCreateWithFlags(&c0->cap_stream, cudaStreamNonBlocking));
@@ -1410,8 +1473,8 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
     for (int i = 0; N && i < count; ++i) {
       pdds_ctx* c = ctxs[i];
       if (N[i])
-        step(pdds::launch_unit_prefix(N[i], c->geo.n, c0->unit_paths, c->d_unit_prefix,
-                                      c->d_path_prefix, &c0->d_scratch->error, s),
+        step(pdds::launch_unit_prefix(N[i], c->geo.n, L.unit_paths, count, L.grid, L.warps(),
+                                      c->d_unit_prefix, c->d_path_prefix, &c0->d_scratch->error, s),
              "unit prefix");
     }
     step(pdds::launch_prob_prefix(c0->d_batch, count, c0->d_prob_prefix, s), "prob prefix");
@@ -1422,7 +1485,7 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
       int calls = 8;
       for (int i = 0; i < count; ++i) calls = std::min(calls, calls_per_check(ctxs[i], dt));
       c0->batch_calls = calls;
-      cap = run_paths(c0, probs[0], c0->d_batch, count, dt, seed, kmax, nullptr, s, sb, max_slots,
+      cap = run_paths(c0, L, probs[0], c0->d_batch, count, dt, seed, kmax, nullptr, s, sb, max_slots,
                       tw, th, c0->coef_id);
       c0->batch_calls = 0;
       c0->timing = timing;

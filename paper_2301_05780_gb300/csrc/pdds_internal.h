@@ -49,8 +49,9 @@ struct ProbDesc {
   const int32_t* slot2csr; // CSR value index per slot, -1 for boundary points
   const int64_t* n_per_knot;      // nullable
   int64_t n_paths;                // uniform budget when n_per_knot == nullptr
-  const int64_t* knot_unit_prefix; // [n+1] units before knot k (per-knot budgets)
-  int64_t units_per_knot;         // uniform budgets
+  const int64_t* knot_unit_prefix; // per-knot budgets: [n+1] units before knot k, then the
+                                  // paths per unit
+  int64_t units_per_knot, unit_paths;  // uniform budgets
   const int64_t* path_prefix;     // [n+1] records before knot k (records mode)
   double* Gval;
   double* b;
@@ -97,7 +98,6 @@ struct KParams {
   int32_t exit_batch;
   int32_t calls_per_check;          // Philox calls (two steps each) between a warp's exit checks
   int64_t total_units;
-  int64_t unit_paths;
   Scratch* scratch;
   PathRecordDev* records;
   uint32_t key0, key1;
@@ -132,8 +132,29 @@ bool path_kernel_has_cv(int coef_id);
 // Control-variate network (pdds_mlp.cu): FP32 theta -> staged image.
 size_t mlp_image_bytes();
 cudaError_t mlp_stage(const float* theta, void* image, cudaStream_t stream);
+// The paths of a work unit for a launch of `paths` paths on `ctas` resident
+// CTAs of `warps` warps, when the caller has set none.  A CTA holds two units
+// at a time, so its lanes stay full only with units of about its lanes, and
+// its last units bound the launch's tail:
+//  - several waves of lanes: 2.5 units per CTA, within one and eight waves of
+//    the CTA's lanes (measured on one GB300, 64-thread CTAs, against 4096:
+//    2.9e5 paths 2.2 -> 0.6 ms; 1.3e6 1.6 -> 0.75; 1.2e6 variable-sigma paths
+//    7.6 -> 5.3; from 5e6 paths on the upper end is within 1 % of the best);
+//  - fewer paths than lanes: one unit per warp, so that every warp has as few
+//    paths as possible (its idle lanes then draw ahead for them).
+__host__ __device__ inline int64_t auto_unit_paths(int64_t paths, int64_t ctas, int64_t warps) {
+  if (paths <= ctas * warps * 32) {
+    const int64_t u = (paths + ctas * warps - 1) / (ctas * warps);
+    return u < 1 ? 1 : u;
+  }
+  const int64_t u = paths * 2 / (5 * ctas), lo = 32 * warps, hi = 256 * warps;
+  return u < lo ? lo : u > hi ? hi : u;
+}
+// Unit and record prefixes of per-knot budgets; unit_paths 0: auto_unit_paths
+// of `share` times the knots' paths (share: problems of the launch).
 // Budgets outside [0, 2^31) count as zero paths and set *err = PDDS_EINVAL.
 cudaError_t launch_unit_prefix(const int64_t* n_per_knot, int64_t n, int64_t unit_paths,
+                               int64_t share, int64_t ctas, int64_t warps,
                                int64_t* knot_unit_prefix, int64_t* path_prefix, int32_t* err,
                                cudaStream_t stream);
 cudaError_t launch_cv_cells(const float* nodes, int nx, int ny, float* cells, cudaStream_t s);

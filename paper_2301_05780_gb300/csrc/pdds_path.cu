@@ -22,38 +22,49 @@ __device__ __forceinline__ int64_t checked_budget(int64_t v, bool& bad) {
   return v;
 }
 
-// Single block: units and records before each knot (exclusive prefix sums).
-// An invalid budget is skipped and recorded as PDDS_EINVAL in *err.
-__global__ void unit_prefix_kernel(const int64_t* __restrict__ N, int64_t n, int64_t C,
-                                   int64_t* __restrict__ up, int64_t* __restrict__ pp,
-                                   int32_t* __restrict__ err) {
-  __shared__ int64_t su[1024], sp[1024];
+// Single block: units and records before each knot (exclusive prefix sums),
+// then the paths per unit.  An invalid budget is skipped and recorded as
+// PDDS_EINVAL in *err.  The records' prefix comes first: its total decides the
+// unit size when the caller has set none (C == 0).
+__global__ void unit_prefix_kernel(const int64_t* __restrict__ N, int64_t n, int64_t C, int64_t share,
+                                   int64_t ctas, int64_t warps, int64_t* __restrict__ up,
+                                   int64_t* __restrict__ pp, int32_t* __restrict__ err) {
+  __shared__ int64_t sum[1024];
   const int t = threadIdx.x, T = blockDim.x;
   const int64_t per = (n + T - 1) / T;
   const int64_t lo = min(n, t * per), hi = min(n, lo + per);
-  int64_t a = 0, b = 0;
+  // inclusive scan of the threads' sums over their knots
+  auto scan = [&](int64_t v) {
+    __syncthreads();
+    sum[t] = v;
+    __syncthreads();
+    for (int o = 1; o < T; o <<= 1) {
+      const int64_t w = t >= o ? sum[t - o] : 0;
+      __syncthreads();
+      sum[t] += w;
+      __syncthreads();
+    }
+    return sum[t] - v;  // exclusive
+  };
   bool bad = false;
-  for (int64_t i = lo; i < hi; ++i) {
-    const int64_t v = checked_budget(N[i], bad);
-    a += (v + C - 1) / C;
-    b += v;
-  }
+  int64_t v = 0;
+  for (int64_t i = lo; i < hi; ++i) v += checked_budget(N[i], bad);
   if (bad) atomicExch(err, (int32_t)PDDS_EINVAL);
-  su[t] = a; sp[t] = b;
-  __syncthreads();
-  for (int o = 1; o < T; o <<= 1) {
-    const int64_t va = t >= o ? su[t - o] : 0, vb = t >= o ? sp[t - o] : 0;
-    __syncthreads();
-    su[t] += va; sp[t] += vb;
-    __syncthreads();
-  }
-  a = su[t] - a; b = sp[t] - b;  // exclusive
+  int64_t before = scan(v);
   for (int64_t i = lo; i < hi; ++i) {
-    up[i] = a; pp[i] = b;
-    const int64_t v = checked_budget(N[i], bad);
-    a += (v + C - 1) / C; b += v;
+    pp[i] = before;
+    before += checked_budget(N[i], bad);
   }
-  if (t == T - 1) { up[n] = su[t]; pp[n] = sp[t]; }
+  const int64_t total = sum[T - 1];
+  if (C == 0) C = auto_unit_paths(share * total, ctas, warps);
+  v = 0;
+  for (int64_t i = lo; i < hi; ++i) v += (checked_budget(N[i], bad) + C - 1) / C;
+  before = scan(v);
+  for (int64_t i = lo; i < hi; ++i) {
+    up[i] = before;
+    before += (checked_budget(N[i], bad) + C - 1) / C;
+  }
+  if (t == T - 1) { up[n] = sum[t]; up[n + 1] = C; pp[n] = total; }
 }
 
 // Units of each problem before it (exclusive prefix over problems).
@@ -161,9 +172,10 @@ cudaError_t set_path_kernel_smem(int coef, bool rec, int cv, bool ext, size_t sm
   return e;
 }
 
-cudaError_t launch_unit_prefix(const int64_t* N, int64_t n, int64_t C, int64_t* up, int64_t* pp,
-                               int32_t* err, cudaStream_t stream) {
-  unit_prefix_kernel<<<1, 1024, 0, stream>>>(N, n, C, up, pp, err);
+cudaError_t launch_unit_prefix(const int64_t* N, int64_t n, int64_t C, int64_t share, int64_t ctas,
+                               int64_t warps, int64_t* up, int64_t* pp, int32_t* err,
+                               cudaStream_t stream) {
+  unit_prefix_kernel<<<1, 1024, 0, stream>>>(N, n, C, share, ctas, warps, up, pp, err);
   return cudaGetLastError();
 }
 
