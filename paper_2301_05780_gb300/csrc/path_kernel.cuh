@@ -15,7 +15,7 @@
 //    exited (exit times are wildly uneven, so lanes never wait for a whole
 //    batch of paths);
 //  - work units are (problem, knot, path range) taken from one global atomic
-//    queue; each CTA keeps a two-stage ring of units in shared memory (knot
+//    queue; each CTA keeps two or three units at a time in shared memory (knot
 //    data, FP64 slot accumulators, TMA-staged coefficient tiles) so warps move
 //    on to the next unit while the stragglers of the previous one finish;
 //  - the warp that completes the last path of a unit flushes its accumulators
@@ -172,12 +172,12 @@ __device__ __forceinline__ void sincos_2pi(float t, float& s, float& c) {
 }
 
 // --------------------------------------------------------------- the stage
-// One entry of a CTA's two-stage unit ring, at the start of its slice of
+// One entry of a CTA's ring of units, at the start of its slice of
 // dynamic shared memory; the FP64 slot accumulators and the coefficient tiles
 // follow it.
 struct alignas(16) Stage {
   // ctrl = state << 32 | next path to hand out.  state = 2q while unit q (the
-  // q-th unit of this CTA) is published, 2q+1 while it is being loaded.  Paths
+  // q-th unit of this stage) is published, 2q+1 while it is being loaded.  Paths
   // are claimed with one 64-bit shared atomic add, so a claim always knows
   // which unit it came from.
   unsigned long long ctrl;
@@ -228,6 +228,11 @@ __device__ __forceinline__ unsigned ctrl_state(const unsigned long long* p) {
   unsigned long long v;
   asm volatile("ld.acquire.cta.shared::cta.b64 %0, [%1];" : "=l"(v) : "r"(smem_u32(p)) : "memory");
   return (unsigned)(v >> 32);
+}
+__device__ __forceinline__ unsigned long long ctrl_word(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.cta.shared::cta.b64 %0, [%1];" : "=l"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
 }
 __device__ __forceinline__ uint64_t global_ns() {
   uint64_t t;
@@ -879,7 +884,7 @@ __device__ int64_t upper_bound_i64(const int64_t* a, int64_t n, int64_t v) {
 }
 
 // Whole warp: take the next unit from the global queue into stage `s` as this
-// CTA's unit number q (or mark the stage terminal).  Returns false on timeout.
+// stage's unit number q (or mark the stage terminal).  Returns false on timeout.
 template <bool EXT>
 __device__ bool load_unit(const Smem& S, int s, int q, const KParams& P, int64_t total_units,
                           int& units_done) {
@@ -1086,8 +1091,8 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
   if (threadIdx.x == 0) {
     s_live = 0;
     s_qempty = 0;
-    for (int s = 0; s < 2; ++s) {
-      S.st(s).ctrl = (unsigned long long)(2u * s + 1u) << 32;  // "loading unit s"
+    for (int s = 0; s < P.stages; ++s) {
+      S.st(s).ctrl = 1ull << 32;  // "loading its unit 0"
       S.st(s).term = 0;
       S.st(s).tma_phase = 0;
       mbar_init(&S.st(s).mbar);
@@ -1096,7 +1101,8 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
   }
   __syncthreads();
   bool ok = true;
-  if (warp < 2) ok = load_unit<EXT>(S, warp, warp, P, total_units, units_done);
+  for (int s = warp; s < P.stages && ok; s += (int)(blockDim.x >> 5))
+    ok = load_unit<EXT>(S, s, 0, P, total_units, units_done);
   __syncthreads();
 
   // lane state
@@ -1118,7 +1124,7 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
   float xk = 0.f, yk = 0.f, bx0 = 0.f, bx1 = 0.f, by0 = 0.f, by1 = 0.f;
   float X = 0.f, Y = 0.f, Sx = 0.f, Z = 0.f, XI = 0.f;
   unsigned long long my_steps = 0, my_paths = 0, my_trunc = 0, my_clamp = 0;
-  int want = 0;  // warp-uniform: unit sequence number the warp takes paths from
+  int from = warp % P.stages;  // warp-uniform: the stage the warp takes paths from
   // EXT: step, its square root and the step cap of the knot the lane's path
   // belongs to, and the Gobet-Menozzi shift per unit of |s| (0: naive exit);
   // the other variants use the launch constants
@@ -1131,13 +1137,20 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
     // ---- hand new paths to idle lanes ----------------------------------
     unsigned idle = __ballot_sync(kFull, !alive);
     for (int guard = 0; idle && guard < 64; ++guard) {
-      Stage& H = S.st(want & 1);
-      const unsigned ss = ctrl_state(&H.ctrl);
-      if ((int)(ss >> 1) > want) { ++want; continue; }      // stage moved past unit `want`
-      if ((ss & 1u) || (int)(ss >> 1) < want) break;       // unit `want` not published yet
-      // A terminal stage only means this load found the queue empty; the other
-      // stage may still hold a unit taken earlier, so move on to it.
-      if (H.term) { ++want; continue; }
+      // Lane s looks at stage s: published, with paths left?  (A hint: the
+      // claim below decides.)  The warp takes the first such stage from its
+      // own starting point on, so that the warps spread over the ring.
+      bool has = false;
+      if (lane < P.stages) {
+        Stage& Q = S.st(lane);
+        const unsigned long long v = ctrl_word(&Q.ctrl);
+        has = !((v >> 32) & 1ull) && !Q.term && (int)(unsigned)v < Q.p_end;
+      }
+      const unsigned avail = __ballot_sync(kFull, has);
+      if (avail == 0) break;
+      const unsigned ahead = avail >> from << from;
+      from = __ffs(ahead ? ahead : avail) - 1;
+      Stage& H = S.st(from);
       const int cnt = __popc(idle);
       const int leader = __ffs(idle) - 1;
       unsigned long long c = 0;
@@ -1145,20 +1158,18 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
       c = __shfl_sync(kFull, c, leader);
       __threadfence_block();
       const unsigned sa = (unsigned)(c >> 32);
-      if (sa & 1u) break;                 // claim landed on a unit being loaded: void
+      if (sa & 1u) continue;              // claim landed on a unit being loaded: void
       const int base = (int)(unsigned)(c & 0xffffffffull);
       const int pend = H.p_end;
       __threadfence_block();
-      if (ctrl_state(&H.ctrl) != sa) {    // unit recycled meanwhile: it was exhausted
-        want = max(want, (int)(sa >> 1) + 1);
-        continue;
-      }
-      want = max(want, (int)(sa >> 1));
+      // unit recycled meanwhile: it was exhausted (a unit with a claimed path
+      // that has not finished cannot be)
+      if (ctrl_state(&H.ctrl) != sa) continue;
       const int got = max(0, min(cnt, pend - base));
       const int rank = __popc(idle & ((1u << lane) - 1u));
       if (!alive && rank < got) {
         alive = true;
-        st = want & 1;
+        st = from;
         p = (uint32_t)(base + rank);
         kk = (uint32_t)H.k;
         tagw = (uint32_t)H.tag;
@@ -1177,7 +1188,6 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
         }
         n = 0; X = 0.f; Y = 0.f; Sx = 0.f; Z = 0.f; XI = 0.f;
       }
-      if (base + cnt >= pend) ++want;     // unit fully handed out
       idle = __ballot_sync(kFull, !alive);
     }
     const unsigned alive_mask = __ballot_sync(kFull, alive);
@@ -1357,11 +1367,10 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
       }
     }
     // warp-aggregated completion counts per stage
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const unsigned m = __ballot_sync(kFull, leaving && !gm_rec && st == s);
-      if (m == 0) continue;
-      __syncwarp();
+    for (unsigned gone = __ballot_sync(kFull, leaving && !gm_rec); gone != 0;) {
+      const int s = __shfl_sync(kFull, st, __ffs(gone) - 1);
+      const unsigned m = __ballot_sync(kFull, st == s) & gone;
+      gone &= ~m;
       __threadfence_block();
       int fin = 0;
       if (lane == 0) {
@@ -1373,7 +1382,7 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
       if (fin) {
         const int q = (int)(ctrl_state(&S.st(s).ctrl) >> 1);
         flush_unit(S, s, P);
-        if (!load_unit<EXT>(S, s, q + 2, P, total_units, units_done)) ok = false;
+        if (!load_unit<EXT>(S, s, q + 1, P, total_units, units_done)) ok = false;
         if (lane == 0) atomicSub(S.live, 1);  // the flushed unit (after the reload reserved)
         __syncwarp();
       }

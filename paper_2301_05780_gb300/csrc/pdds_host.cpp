@@ -429,7 +429,7 @@ int64_t default_kmax(const pdds_ctx* c, double dt) {
 
 // The shape of one path-kernel launch.
 struct LaunchPlan {
-  int cv = 0, block = 0, grid = 0, exit_batch = 0;
+  int cv = 0, block = 0, grid = 0, exit_batch = 0, stages = 2;
   size_t smem = 0;
   int64_t unit_paths = 0;  // 0: auto_unit_paths
   int64_t warps() const { return block / 32; }
@@ -451,9 +451,10 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
   if (L.cv == 1 && c->net_engine == PDDS_NET_TCGEN05) L.cv = 3;
   // network kernels keep the staged network at the start of dynamic shared
   // memory (the tcgen05 kernel: its swizzled operand tiles)
-  L.smem = 2 * sbytes + (L.cv == 1   ? round_up(pdds::mlp_image_bytes(), 128)
-                         : L.cv == 3 ? pdds::net_smem_bytes()
-                                     : 0);
+  const size_t net = L.cv == 1   ? round_up(pdds::mlp_image_bytes(), 128)
+                     : L.cv == 3 ? pdds::net_smem_bytes()
+                                 : 0;
+  L.smem = 2 * sbytes + net;
   CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, L.smem));
   int per_sm = 0;
   if (L.cv == 3) {
@@ -479,6 +480,26 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
   }
   // tcgen05 kernel: 96 TMEM columns per CTA, 512 per SM
   if (L.cv == 3) per_sm = std::min(per_sm, 512 / 96);
+  if (L.cv != 3) {
+    // A unit's stage is free again only when its last path has left, so with
+    // two stages the lanes run dry where units are short (per-knot budgets,
+    // wide stencils): a third one, where the resident CTAs stay and, with the
+    // tabulated control variate, the L1 cache keeps 60 KB for the table.  One
+    // GB300, two / three / four stages: RBF stencils 9.6 / 8.9 / 8.9 ms, the
+    // paper's production run 45.3 / 42.1 / 43.1, batch of 16 461 / 455 / 455;
+    // L1 below 50 KB: 56.
+    const size_t three = 3 * sbytes + net;
+    if (three * per_sm <= (L.cv == 2 ? 160 : 227) * 1024) {
+      int ctas = 0;
+      CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, three));
+      CK(c, pdds::path_kernel_occupancy(coef_id, rec, L.cv, ext, L.block, three, &ctas));
+      if (ctas >= per_sm) {
+        L.stages = 3;
+        L.smem = three;
+      }
+    }
+    CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, L.smem));
+  }
   L.grid = c->num_sms * per_sm;
   // (the warpgroup kernel steps 128 paths at a time, however few are left)
   L.unit_paths = c->auto_unit && L.cv != 3 ? 0 : c->unit_paths;
@@ -517,6 +538,7 @@ pdds_status run_paths(pdds_ctx* c, const LaunchPlan& L, const ProbDesc& p0, cons
   kp.tile_w = tile_w;
   kp.tile_h = tile_h;
   kp.stage_bytes = (int)sbytes;
+  kp.stages = L.stages;
   kp.mixed = rec_gm != nullptr ? 1 : 0;
   kp.records_gm = rec_gm;
   // a wait may outlast the slowest path of a unit: K_max steps at ~4 us

@@ -108,7 +108,7 @@ struct KParams {
   int32_t tile_w, tile_h;  // TABLE tile (nodes)
   int32_t stage_bytes;     // bytes per stage in dynamic shared memory
   int32_t mixed;           // records kernels with the extended exit: 1 = mixed GM/EM run
-  int32_t pad_;
+  int32_t stages;          // stages of a CTA's unit ring (<= 32)
   PathRecordDev* records_gm;  // mixed run: the Gobet-Menozzi exit of each path
   uint64_t wait_ns;        // bound on any device-side wait
   const void* mlp;         // staged control-variate network (MlpSmem), or nullptr
