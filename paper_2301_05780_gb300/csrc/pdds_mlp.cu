@@ -18,6 +18,7 @@
 
 #include "pdds.h"
 #include "pdds_internal.h"
+#include "device_scratch.h"
 #include "mlp_train.h"
 #include "pdds_mlp.cuh"
 
@@ -538,8 +539,9 @@ pdds_status train_impl(int engine, const char* name, float* theta, const float* 
   const size_t fbytes = 9 * kMlpParams * sizeof(float);
   const size_t sbytes = (fbytes + 15) / 16 * 16;
   const size_t bytes = sbytes + sizeof(TrainState) + (size_t)steps * sizeof(double);
-  char* buf = nullptr;
-  MCK(cudaMalloc(reinterpret_cast<void**>(&buf), bytes));
+  DeviceScratch scratch;
+  MCK(scratch.get(bytes));
+  char* const buf = static_cast<char*>(scratch.ptr());
   float* f = reinterpret_cast<float*>(buf);
   TrainArgs a{};
   a.theta = theta;
@@ -606,7 +608,8 @@ pdds_status train_impl(int engine, const char* name, float* theta, const float* 
     return cudaStreamSynchronize(s);
   };
   cudaError_t e = run();
-  cudaFree(buf);
+  // (also after a failure: the buffer goes back only when nothing uses it)
+  if (e != cudaSuccess) (void)cudaStreamSynchronize(s);
   if (e != cudaSuccess) return mlp_cuda(e, name);
   return PDDS_OK;
 }
@@ -632,8 +635,9 @@ extern "C" pdds_status pdds_mlp_eval(const float* theta, const float* xy, int64_
     return mlp_fail(PDDS_EINVAL, "mlp_eval: NULL pointer or npts < 1");
   (void)cudaGetLastError();
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  void* img = nullptr;
-  MCK(cudaMalloc(&img, sizeof(MlpSmem)));
+  DeviceScratch scratch;
+  MCK(scratch.get(sizeof(MlpSmem)));
+  void* const img = scratch.ptr();
   cudaError_t e = mlp_stage(theta, img, s);
   if (e == cudaSuccess) {
     const int64_t blocks = (npts + 255) / 256;
@@ -641,8 +645,8 @@ extern "C" pdds_status pdds_mlp_eval(const float* theta, const float* xy, int64_
                                                       npts, v, grad_xy);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(img);
+  const cudaError_t done = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = done;
   if (e != cudaSuccess) return mlp_cuda(e, "mlp_eval");
   return PDDS_OK;
 }

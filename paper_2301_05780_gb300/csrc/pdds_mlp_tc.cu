@@ -1,20 +1,31 @@
 // The network v_theta (2 -> 64 -> 64 -> 1, SiLU; Eq. 11, 37-39) on the
 // fifth-generation tensor cores: v and grad v at many points, tile by tile.
 //
-// A CTA of two warpgroups (256 threads); each warpgroup takes its own tiles of
-// 128 points, thread t of the group owning point t of the tile (TMEM lane t),
-// with its own operand buffers, mbarrier and TMEM columns, and synchronises on
-// its own named barrier, so the two groups' MMAs and SIMT work overlap.
-// Per tile:
-//   layer 1 (FP32 SIMT)    a1 = W1 x + b1, h1 = SiLU(a1), SiLU'(a1) kept
-//   forward (tcgen05)      D1 = h1 W2^T            [128 x 64], TMEM cols 0-63
-//   output  (FP32 SIMT)    a2 = D1 + b2, v = w3 . SiLU(a2) + b3,
+// A CTA of four warpgroups (512 threads), one per SM; each warpgroup takes its
+// own tiles of 128 points, thread t of the group owning point t of the tile
+// (TMEM lane t), with its own operand buffer, mbarrier and TMEM columns, and
+// synchronises on its own named barrier, so the groups' MMAs and SIMT work
+// overlap.  Per tile:
+//   layer 1 (FP32 SIMT)    a1 = W1 x + b1, h1 = SiLU(a1); SiLU'(a1) into TMEM
+//   forward (tcgen05)      D = h1 W2^T              [128 x 64], TMEM
+//   output  (FP32 SIMT)    a2 = D + b2, v = w3 . SiLU(a2) + b3,
 //                          g2 = w3 * SiLU'(a2) = dv / da2
-//   backward (tcgen05)     D2 = g2 W2               [128 x 64], TMEM cols 64-127
-//   input gradient (SIMT)  grad v = W1^T (D2 * SiLU'(a1))
+//   backward (tcgen05)     D = g2 W2                [128 x 64], TMEM
+//   input gradient (SIMT)  grad v = W1^T (D * SiLU'(a1))
 // h1 and g2 are the M x K operand (K-major, 128-byte swizzle), W2 and W2^T
 // the N x K operands, staged once per CTA.  Every product is the 3xTF32 split
 // (tc_sm103.cuh), so v and grad v carry FP32 rounding only.
+//
+// What bounds it: the SiLUs (two special-function operations and about ten
+// instructions per unit, 128 units per point), which only enough warps keep
+// flowing through a tile's chain of products.  So the operand goes through one
+// 32-unit half buffer (hi and lo: 32 KB per group instead of 64): the half's
+// MMA runs while the other half's units are computed in registers; SiLU'(a1)
+// waits in TMEM instead of 64 registers; the units run in packed FP32 pairs.
+// That makes 16 warps per SM instead of 8, at two thirds of the instructions
+// (55 per point and warp lane instead of 82).  One GB300, 1.59e6 points: kernel
+// 330 -> 190 us, the call with its kept scratch 525 -> 245 us; 1,000 points 211
+// -> 48 us.  3xTF32 at N = 64 keeps the tensor pipe busy for about 115 us of it.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -23,6 +34,7 @@
 
 #include "pdds.h"
 #include "pdds_internal.h"
+#include "device_scratch.h"
 #include "tc_sm103.cuh"
 
 namespace pdds {
@@ -32,12 +44,14 @@ constexpr int kH = 64;    // hidden width
 constexpr int kTP = 128;  // points per tile = MMA M
 constexpr int kOffW2 = 192, kOffB1 = 128, kOffB2 = 4288, kOffW3 = 4352, kOffB3 = 4416;
 
-constexpr int kGroups = 2;  // warpgroups per CTA
+constexpr int kGroups = 4;   // warpgroups per CTA
+constexpr int kHalf = kH / 2;  // units per operand buffer
+constexpr unsigned kColsGroup = 128;  // TMEM per group: D (64 columns), SiLU'(a1) (64)
 
 struct alignas(1024) EvalTcSmem {
-  float B1[2][kH * kH];           // W2 as N = out x K = in, hi and lo parts
-  float B2[2][kH * kH];           // W2^T as N = in x K = out
-  float A[kGroups][2][kTP * kH];  // per group: h1, then g2 (M = point x K = unit)
+  float B1[2][kH * kH];              // W2 as N = out x K = in, hi and lo parts
+  float B2[2][kH * kH];              // W2^T as N = in x K = out
+  float A[kGroups][2][kTP * kHalf];  // per group: half of h1 or g2 (M = point x K = unit)
   float w1x[kH], w1y[kH], b1[kH], b2[kH], w3[kH];
   float b3;
   unsigned long long mbar[kGroups];
@@ -45,36 +59,55 @@ struct alignas(1024) EvalTcSmem {
 };
 constexpr size_t kEvalTcSmemBytes = sizeof(EvalTcSmem) + 1024;  // + alignment slack
 
-// 1 / (1 + e^-a) with the fast reciprocal-based division (a few ulp; 0 when
-// e^-a overflows)
-__device__ __forceinline__ float logistic(float a) { return __fdividef(1.0f, 1.0f + __expf(-a)); }
+__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
+
+// 1 / (1 + e^-a) from the hardware exponential and reciprocal (a few ulp; 0
+// when e^-a overflows; where e^-a would be denormal the sum is 1 either way)
+__device__ __forceinline__ float2 logistic2(float2 a) {
+  const float2 t = mul2(a, f2(-1.4426950408889634f, -1.4426950408889634f));
+  float ex, ey, rx, ry;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(t.x));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ey) : "f"(t.y));
+  const float2 y = add2(f2(ex, ey), f2(1.0f, 1.0f));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rx) : "f"(y.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ry) : "f"(y.y));
+  return f2(rx, ry);
+}
+// SiLU'(a) = sg (1 + a (1 - sg)) from the logistic sg
+__device__ __forceinline__ float2 dsilu2(float2 a, float2 sg) {
+  const float2 m = add2(f2(1.0f, 1.0f), f2(-sg.x, -sg.y));
+  return mul2(sg, fma2(a, m, f2(1.0f, 1.0f)));
+}
 __device__ __forceinline__ void group_sync(int g) {
   asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kTP) : "memory");
 }
 
-__device__ __forceinline__ void put_split(float* hi_base, float* lo_base, int off_bytes, float4 v) {
-  float4 h = make_float4(tc::tf32_hi(v.x), tc::tf32_hi(v.y), tc::tf32_hi(v.z), tc::tf32_hi(v.w));
-  float4 l = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
+// Units 4c .. 4c + 3 of this point's half into the operand buffers, split.
+__device__ __forceinline__ void put_split(float* hi_base, float* lo_base, int off_bytes, float2 v,
+                                          float2 w) {
+  const float4 h = make_float4(tc::tf32_hi(v.x), tc::tf32_hi(v.y), tc::tf32_hi(w.x), tc::tf32_hi(w.y));
+  const float2 l0 = add2(v, f2(-h.x, -h.y)), l1 = add2(w, f2(-h.z, -h.w));
   *reinterpret_cast<float4*>(reinterpret_cast<char*>(hi_base) + off_bytes) = h;
-  *reinterpret_cast<float4*>(reinterpret_cast<char*>(lo_base) + off_bytes) = l;
+  *reinterpret_cast<float4*>(reinterpret_cast<char*>(lo_base) + off_bytes) =
+      make_float4(l0.x, l0.y, l1.x, l1.y);
 }
 
-// D (TMEM, 64 columns at d) = A B^T with the 3xTF32 split: 3 x 8 K-steps.
-__device__ __forceinline__ void mma_3xtf32(unsigned d, const float* const (&A)[2],
-                                           const float* const (&B)[2]) {
+// D (TMEM, 64 columns at d) [+]= A B^T over the 32 units of half `hf` with the
+// 3xTF32 split: 3 x 4 K-steps.
+__device__ __forceinline__ void mma_half(unsigned d, unsigned a_hi, unsigned a_lo, unsigned b_hi,
+                                         unsigned b_lo, int hf) {
   constexpr uint32_t idesc = tc::idesc_tf32(kTP, kH);
-  bool acc = false;
 #pragma unroll
-  for (int pr = 0; pr < 3; ++pr) {
-    const int ia = pr == 2 ? 1 : 0, ib = pr == 1 ? 1 : 0;  // hi hi, hi lo, lo hi
+  for (int pr = 0; pr < 3; ++pr) {  // hi hi, hi lo, lo hi
+    const unsigned a = pr == 2 ? a_lo : a_hi, b = (pr == 1 ? b_lo : b_hi) + hf * kH * 128;
 #pragma unroll
-    for (int kk = 0; kk < 8; ++kk) {
-      const unsigned ka = (kk >> 2) * kTP * 128 + (kk & 3) * 32;
-      const unsigned kb = (kk >> 2) * kH * 128 + (kk & 3) * 32;
-      tc::mma_tf32(d, tc::sdesc_k128(tc::smem_addr(A[ia]) + ka),
-                   tc::sdesc_k128(tc::smem_addr(B[ib]) + kb), idesc, acc);
-      acc = true;
-    }
+    for (int kk = 0; kk < 4; ++kk)
+      tc::mma_tf32(d, tc::sdesc_k128(a + kk * 32), tc::sdesc_k128(b + kk * 32), idesc,
+                   hf > 0 || pr > 0 || kk > 0);
   }
 }
 
@@ -107,113 +140,130 @@ __global__ void __launch_bounds__(kGroups * kTP, 1)
     S.b3 = theta[kOffB3];
     for (int q = 0; q < kGroups; ++q) tc::mbar_init(&S.mbar[q]);
   }
-  if (warp == 0) tc::tmem_alloc(&S.tmem, 128 * kGroups);
+  if (warp == 0) tc::tmem_alloc(&S.tmem, kColsGroup * kGroups);
   tc::fence_async_smem();
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   // group g: TMEM columns [128 g, 128 g + 128); its warps read lanes 32 (warp % 4) ..
-  const unsigned tm = S.tmem + 128u * g;
+  const unsigned tm = S.tmem + kColsGroup * g, tm_s1 = tm + kH;
   const unsigned lane = (unsigned)((warp & 3) * 32) << 16;
   float* const A0 = S.A[g][0];
   float* const A1 = S.A[g][1];
-  const float* const Aop[2] = {A0, A1};
-  const float* const B1op[2] = {S.B1[0], S.B1[1]};
-  const float* const B2op[2] = {S.B2[0], S.B2[1]};
   unsigned long long* const mbar = &S.mbar[g];
   unsigned phase = 0;
   bool ok = true;
-  for (int64_t tile = (int64_t)kGroups * blockIdx.x + g; tile * kTP < npts;
-       tile += (int64_t)kGroups * gridDim.x) {
-    const int64_t p = tile * kTP + t;
+  // The operand half in the buffers is complete: its product, by one thread.
+  auto issue = [&](const float (&B)[2][kH * kH], int hf) {
+    tc::fence_async_smem();
+    tc::fence_before();
+    group_sync(g);
+    if (t == 0) {
+      tc::fence_after();
+      mma_half(tm, tc::smem_addr(A0), tc::smem_addr(A1), tc::smem_addr(B[0]), tc::smem_addr(B[1]), hf);
+      tc::commit(mbar);
+    }
+  };
+  auto wait = [&] {
+    ok = tc::mbar_wait(mbar, phase, 2000000000ull) && ok;
+    phase ^= 1u;
+    tc::fence_after();
+  };
+  const int64_t stride = (int64_t)kGroups * gridDim.x * kTP;
+  int64_t p = ((int64_t)g * gridDim.x + blockIdx.x) * kTP + t;
+  auto point = [&](int64_t q) { return q < npts ? f2(xy[2 * q], xy[2 * q + 1]) : f2(0.f, 0.f); };
+  float2 next = point(p);  // one tile ahead
+  for (; p - t < npts; p += stride) {
     const bool valid = p < npts;
-    const float x = valid ? xy[2 * p] : 0.f, y = valid ? xy[2 * p + 1] : 0.f;
-    // layer 1: h1 into the A tile, SiLU'(a1) kept
-    float s1[kH];
+    const float x = next.x, y = next.y;
+    next = point(p + stride);
+    // layer 1, 16 units from u0 on: h into h[], SiLU' into TMEM
+    auto layer1 = [&](int u0, float2* h) {
+      float s1[16];
 #pragma unroll
-    for (int c = 0; c < kH / 4; ++c) {
-      float h[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int u = 4 * c + j;
-        const float a = fmaf(S.w1x[u], x, fmaf(S.w1y[u], y, S.b1[u]));
-        const float sg = logistic(a);
-        h[j] = a * sg;
-        s1[u] = sg * (1.0f + a * (1.0f - sg));
+      for (int j = 0; j < 16; j += 2) {
+        const int u = u0 + j;
+        const float2 a = fma2(ld2(&S.w1x[u]), f2(x, x), fma2(ld2(&S.w1y[u]), f2(y, y), ld2(&S.b1[u])));
+        const float2 sg = logistic2(a);
+        h[j / 2] = mul2(a, sg);
+        const float2 d = dsilu2(a, sg);
+        s1[j] = d.x;
+        s1[j + 1] = d.y;
       }
-      put_split(A0, A1, tc::swz_chunk(t, c, kTP), make_float4(h[0], h[1], h[2], h[3]));
-    }
-    tc::fence_async_smem();
-    tc::fence_before();
-    group_sync(g);
-    if (t == 0) {
-      tc::fence_after();
-      mma_3xtf32(tm, Aop, B1op);
-      tc::commit(mbar);
-    }
-    ok = tc::mbar_wait(mbar, phase, 2000000000ull) && ok;
-    phase ^= 1u;
-    tc::fence_after();
-    // a2 -> v and g2 = w3 SiLU'(a2) (into the A tile: the forward MMA is done)
-    float vs = S.b3;
+      tc::tmem_st16(tm_s1 + lane + u0, s1);
+    };
+    auto put16 = [&](int c0, const float2* h) {  // chunks c0 .. c0 + 3 of the half
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      float d[32];
-      tc::tmem_ld32(tm + lane + 32 * half, d);
+      for (int c = 0; c < 4; ++c)
+        put_split(A0, A1, tc::swz_chunk(t, c0 + c, kTP), h[2 * c], h[2 * c + 1]);
+    };
+    float2 h[16];
+    layer1(0, h);
+    put16(0, h);
+    layer1(16, h);
+    put16(4, h);
+    issue(S.B1, 0);
+    layer1(kHalf, h);
+    layer1(kHalf + 16, h + 8);
+    wait();
+    put16(0, h);
+    put16(4, h + 8);
+    tc::st_wait();
+    issue(S.B1, 1);
+    wait();
+    // a2 -> v and g2 = w3 SiLU'(a2), 32 outputs from o0 on
+    float2 vs = f2(S.b3, 0.f);
+    auto output = [&](int o0, float (&d)[32], float2* gg) {
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        float g[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int o = 32 * half + 4 * c + j;
-          const float a = d[4 * c + j] + S.b2[o];
-          const float sg = logistic(a);
-          vs = fmaf(S.w3[o], a * sg, vs);
-          g[j] = S.w3[o] * (sg * (1.0f + a * (1.0f - sg)));
-        }
-        put_split(A0, A1, tc::swz_chunk(t, 8 * half + c, kTP),
-                  make_float4(g[0], g[1], g[2], g[3]));
+      for (int j = 0; j < 32; j += 2) {
+        const int o = o0 + j;
+        const float2 a = add2(f2(d[j], d[j + 1]), ld2(&S.b2[o]));
+        const float2 w = ld2(&S.w3[o]);
+        const float2 sg = logistic2(a);
+        vs = fma2(w, mul2(a, sg), vs);
+        gg[j / 2] = mul2(w, dsilu2(a, sg));
       }
-    }
-    tc::fence_async_smem();
-    tc::fence_before();
-    group_sync(g);
-    if (t == 0) {
-      tc::fence_after();
-      mma_3xtf32(tm + 64, Aop, B2op);
-      tc::commit(mbar);
-    }
-    ok = tc::mbar_wait(mbar, phase, 2000000000ull) && ok;
-    phase ^= 1u;
-    tc::fence_after();
+    };
+    float d[32];
+    tc::tmem_ld32(tm + lane, d);
+    output(0, d, h);
+    put16(0, h);
+    put16(4, h + 8);
+    tc::tmem_ld32(tm + lane + kHalf, d);  // before the backward product takes D's place
+    issue(S.B2, 0);
+    output(kHalf, d, h);
+    wait();
+    put16(0, h);
+    put16(4, h + 8);
+    issue(S.B2, 1);
+    wait();
     // grad v = W1^T (dh1 * SiLU'(a1))
-    float gx = 0.f, gy = 0.f;
+    float2 gx = f2(0.f, 0.f), gy = f2(0.f, 0.f);
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      float d[32];
-      tc::tmem_ld32(tm + lane + 64 + 32 * half, d);
+    for (int q = 0; q < 4; ++q) {
+      float dh[16], s1[16];
+      tc::tmem_ld16x2(tm + lane + 16 * q, tm_s1 + lane + 16 * q, dh, s1);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        const int u = 32 * half + j;
-        const float da = d[j] * s1[u];
-        gx = fmaf(da, S.w1x[u], gx);
-        gy = fmaf(da, S.w1y[u], gy);
+      for (int j = 0; j < 16; j += 2) {
+        const int u = 16 * q + j;
+        const float2 da = mul2(f2(dh[j], dh[j + 1]), f2(s1[j], s1[j + 1]));
+        gx = fma2(da, ld2(&S.w1x[u]), gx);
+        gy = fma2(da, ld2(&S.w1y[u]), gy);
       }
     }
     if (valid) {
-      if (v) v[p] = vs;
-      gxy[2 * p] = gx;
-      gxy[2 * p + 1] = gy;
+      if (v) v[p] = vs.x + vs.y;
+      gxy[2 * p] = gx.x + gx.y;
+      gxy[2 * p + 1] = gy.x + gy.y;
     }
-    // TMEM reads of this tile done before the group's next MMAs
-    tc::fence_before();
-    group_sync(g);
+    // (the next product into D follows the group's next barrier, so every
+    // thread has read its columns by then)
   }
   tc::fence_before();
   __syncthreads();
   if (warp == 0) {
     tc::fence_after();
-    tc::tmem_dealloc(S.tmem, 128 * kGroups);
+    tc::tmem_dealloc(S.tmem, kColsGroup * kGroups);
   }
   if (!ok && t == 0) atomicExch(err, (int)PDDS_ETIMEOUT);
 }
@@ -235,22 +285,26 @@ extern "C" pdds_status pdds_mlp_eval_tc(const float* theta, const float* xy, int
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int* d_err = nullptr;
-  if (e == cudaSuccess) e = cudaMalloc(&d_err, sizeof(int));
+  DeviceScratch scratch;
+  if (e == cudaSuccess) e = scratch.get(sizeof(int));
+  d_err = static_cast<int*>(scratch.ptr());
   if (e == cudaSuccess) e = cudaMemsetAsync(d_err, 0, sizeof(int), s);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(mlp_eval_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kEvalTcSmemBytes);
   if (e == cudaSuccess) {
     const int64_t tiles = (npts + kTP - 1) / kTP;
-    const int grid = (int)std::min<int64_t>((tiles + kGroups - 1) / kGroups, sms);
+    // a tile per SM first, then a second group's, and so on
+    const int grid = (int)std::min<int64_t>(tiles, sms);
     mlp_eval_tc_kernel<<<grid, kGroups * kTP, kEvalTcSmemBytes, s>>>(theta, xy, npts, v, grad_xy,
                                                                       d_err);
     e = cudaGetLastError();
   }
   int herr = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(d_err);
+  // also after a failure: the buffer goes back only when nothing uses it
+  const cudaError_t done = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = done;
   if (e != cudaSuccess) {
     set_global_error(std::string("mlp_eval_tc: ") + cudaGetErrorString(e));
     return PDDS_ECUDA;
