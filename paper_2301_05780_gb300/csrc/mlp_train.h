@@ -12,7 +12,7 @@ constexpr int kOffW1 = 0, kOffB1 = 128, kOffW2 = 192, kOffB2 = 4288, kOffW3 = 43
 
 // Step state of a training run (device, zeroed before the first step).
 struct TrainState {
-  unsigned count;  // CTAs done with the current launch
+  unsigned count;  // CTAs done with the current launch (persistent: arrivals at the barrier)
   int t;           // index of the next launch
   double p1, p2;   // beta1^t, beta2^t for launch t >= 1
 };
@@ -31,6 +31,8 @@ struct TrainArgs {
   TrainState* st;
   int steps;
   float lr, beta1, beta2, eps;
+  int grad_stride;  // floats between the rotating gradient buffers
+  int persistent;   // 1: all steps in one cooperative launch
 };
 
 // The tensor-core training kernel (pdds_mlp_train_tc.cu): its function, grid,

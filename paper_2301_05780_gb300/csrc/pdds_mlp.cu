@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kTrainThreads, 2) mlp_train_kernel(const Train
   } else if (grad_pass || blockIdx.x == 0) {
     // Adam update t from the parameters, moments and gradient of launch t - 1
     const int rd = ((t - 1) & 1) * kMlpParams, wr = (t & 1) * kMlpParams;
-    const float* gp = A.grad + ((t - 1) % 3) * kMlpParams;
+    const float* gp = A.grad + ((t - 1) % 3) * A.grad_stride;
     const float c1 = (float)(1.0 - __ldcg(&A.st->p1)), c2 = (float)(1.0 - __ldcg(&A.st->p2));
     float g[kPer], mo[kPer], vo[kPer], to[kPer];
 #pragma unroll
@@ -157,12 +157,12 @@ __global__ void __launch_bounds__(kTrainThreads, 2) mlp_train_kernel(const Train
   }
   if (ADAM && blockIdx.x == 0) {
     // clear the gradient buffer launch t + 1 accumulates into (last read by t - 1)
-    float* gz = A.grad + ((t + 1) % 3) * kMlpParams;
+    float* gz = A.grad + ((t + 1) % 3) * A.grad_stride;
     for (int i = tid; i < kMlpParams; i += kTrainThreads) gz[i] = 0.f;
   }
   __syncthreads();
   if (grad_pass) {
-  float* gacc = A.grad + (ADAM ? (t % 3) * kMlpParams : 0);
+  float* gacc = A.grad + (ADAM ? (t % 3) * A.grad_stride : 0);
   const int c0 = 4 * tx, r0 = kMR * ty;
   float dW2[kMR][4] = {};                          // o = r0 + i, u = c0 + j
   float gw1x[4] = {}, gw1y[4] = {}, gb1[4] = {};  // u = c0 + j
@@ -305,10 +305,20 @@ __global__ void __launch_bounds__(kTrainThreads, 2) mlp_train_kernel(const Train
     __syncthreads();  // h1 and g2 are overwritten by the next tile
   }
   // ---- the CTA's partial gradient into grad
+  // (dW2 as four-float reductions where the buffer is 16-byte aligned, as the
+  // trainer's own are: a quarter of the L2 transactions, which took longer than
+  // the products)
+  const bool vec = (reinterpret_cast<uintptr_t>(gacc) & 15) == 0;
 #pragma unroll
-  for (int i = 0; i < kMR; ++i)
+  for (int i = 0; i < kMR; ++i) {
+    float* to = gacc + kOffW2 + (r0 + i) * kMlpHidden + c0;
+    if (vec) {
+      atomicAdd(reinterpret_cast<float4*>(to), make_float4(dW2[i][0], dW2[i][1], dW2[i][2], dW2[i][3]));
+    } else {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) atomicAdd(gacc + kOffW2 + (r0 + i) * kMlpHidden + c0 + j, dW2[i][j]);
+      for (int j = 0; j < 4; ++j) atomicAdd(to + j, dW2[i][j]);
+    }
+  }
   // column sums: the two row groups of a warp (lanes 0-15, 16-31) by a
   // shuffle, then over the warps (staged over h1 and g2)
   constexpr int kWarps = kTrainThreads / 32;
@@ -536,7 +546,9 @@ pdds_status train_impl(int engine, const char* name, float* theta, const float* 
   MCK(train_config(engine, true, npts, &fn, &grid, &threads, &smem));
   // scratch: three gradients and two each of theta, m, v (FP32), the step
   // state, the loss history
-  const size_t fbytes = 9 * kMlpParams * sizeof(float);
+  // (gradients on a 16-byte stride: the tensor-core kernel adds four at a time)
+  constexpr int kGradStride = (kMlpParams + 3) / 4 * 4;
+  const size_t fbytes = (3 * kGradStride + 6 * kMlpParams) * sizeof(float);
   const size_t sbytes = (fbytes + 15) / 16 * 16;
   const size_t bytes = sbytes + sizeof(TrainState) + (size_t)steps * sizeof(double);
   DeviceScratch scratch;
@@ -551,9 +563,10 @@ pdds_status train_impl(int engine, const char* name, float* theta, const float* 
   a.scale = 2.0f / (float)npts;
   a.inv_n = 1.0 / (double)npts;
   a.grad = f;
-  a.th2 = f + 3 * kMlpParams;
-  a.m2 = f + 5 * kMlpParams;
-  a.v2 = f + 7 * kMlpParams;
+  a.grad_stride = kGradStride;
+  a.th2 = f + 3 * kGradStride;
+  a.m2 = a.th2 + 2 * kMlpParams;
+  a.v2 = a.m2 + 2 * kMlpParams;
   a.st = reinterpret_cast<TrainState*>(buf + sbytes);
   a.loss = reinterpret_cast<double*>(buf + sbytes + sizeof(TrainState));
   a.steps = steps;
@@ -564,6 +577,22 @@ pdds_status train_impl(int engine, const char* name, float* theta, const float* 
   auto run = [&]() -> cudaError_t {
     cudaError_t r = cudaMemsetAsync(buf, 0, bytes, s);
     if (r != cudaSuccess) return r;
+    if (engine == 1) {
+      // tensor-core engine: every step in one cooperative launch while the
+      // device holds all its CTAs at once, else launch by launch as below
+      TrainArgs pa = a;
+      pa.persistent = 1;
+      void* args[] = {&pa};
+      r = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(threads), args, smem, s);
+      if (r != cudaErrorCooperativeLaunchTooLarge) {
+        if (r == cudaSuccess && loss_history_host)
+          r = cudaMemcpyAsync(loss_history_host, a.loss, steps * sizeof(double),
+                              cudaMemcpyDeviceToHost, s);
+        if (r == cudaSuccess) r = cudaStreamSynchronize(s);
+        return r;
+      }
+      (void)cudaGetLastError();
+    }
     // steps + 1 launches (gradients 0..steps-1, updates 1..steps) run as a
     // CUDA graph of 64 identical launches replayed on a private stream (the
     // launch index is read on the device; launches past the last return at

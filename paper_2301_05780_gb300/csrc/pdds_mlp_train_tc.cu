@@ -20,10 +20,16 @@
 // thread also writes its column of the unit-major tiles (g2^T, g1^T, h2^T,
 // h1^T, x, y, 1, dv).  All tiles are K-major BF16 with the 128-byte swizzle.
 //
-// The Adam step, the rotation of the gradient, parameter and moment buffers
-// across launches and the step counter are those of the FP32 kernel
-// (pdds_mlp.cu); only the gradient differs, by the BF16 rounding of the
-// products' operands.  Waits on the tensor core are bounded (2 s); a wait
+// The Adam step and the rotation of the gradient, parameter and moment buffers
+// across steps are those of the FP32 kernel (pdds_mlp.cu); only the gradient
+// differs, by the BF16 rounding of the products' operands.  While the CTAs
+// are all resident (one tile each at the sizes of a warm-up fit) the steps of
+// a run are one cooperative launch with a grid barrier per step instead of a
+// launch per step.  One GB300, per step at 11,241 / 113,665 points: 21.3 / 58.1 us
+// with a launch per step and the gradient added one float at a time, 14.9 / 31.5
+// with four-float reductions (a CTA's 4,417 reductions were 4,417 L2
+// transactions), 13.4 / 31.5 in one launch (more than one tile per SM: launch
+// by launch).  Waits on the tensor core are bounded (2 s); a wait
 // that runs out turns the step's loss into NaN.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -66,6 +72,7 @@ struct alignas(1024) TrainTcSmem {
   double red_loss[kThreads / 32];
   unsigned long long mbar;
   unsigned tmem;
+  int met;
 };
 constexpr size_t kTrainTcSmemBytes = sizeof(TrainTcSmem) + 1024;  // + alignment slack
 
@@ -133,10 +140,42 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int kPer = (kMlpParams + kThreads - 1) / kThreads;
   int t = 0;
+  double p1 = 1.0, p2 = 1.0;  // beta1^t, beta2^t
   if constexpr (ADAM) {
-    t = __ldcg(&A.st->t);
-    if (t > A.steps) return;  // a launch queued past the last one
+    if (!A.persistent) {
+      t = __ldcg(&A.st->t);
+      if (t > A.steps) return;  // a launch queued past the last one
+      p1 = __ldcg(&A.st->p1);
+      p2 = __ldcg(&A.st->p2);
+    }
   }
+  // rows 64-79 of the gradient B tile (x, y and 1 are rewritten per tile, the
+  // rest stay zero) and the whole dv tile
+  for (int i = tid; i < 2 * 16 * 128 / 16; i += kThreads) {
+    const int a = i / 128, w = i % 128;  // atom column, 16-byte word within rows 64-79
+    *reinterpret_cast<uint4*>(reinterpret_cast<char*>(S.GB) + a * kBR * 128 + 8 * 1024 + 16 * w) =
+        make_uint4(0u, 0u, 0u, 0u);
+  }
+  for (int i = tid; i < kVR * kTT * 2 / 16; i += kThreads)
+    *reinterpret_cast<uint4*>(reinterpret_cast<char*>(S.DV) + 16 * i) = make_uint4(0u, 0u, 0u, 0u);
+  if (tid == 0) tc::mbar_init(&S.mbar);
+  if (warp == 0) tc::tmem_alloc(&S.tmem, kTmemCols);
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  // warpgroup g takes hidden units [32 g, 32 g + 32) of every point; thread
+  // pl of the group owns point pl of the tile and TMEM lane pl
+  const int g = tid / kTT, pl = tid % kTT;
+  const unsigned tm = S.tmem, tl = (unsigned)((warp & 3) * 32) << 16;
+  const unsigned sP = tc::smem_addr(S.P), sGA = tc::smem_addr(S.GA), sGB = tc::smem_addr(S.GB);
+  const unsigned sDV = tc::smem_addr(S.DV);
+  unsigned phase = 0;
+  bool ok = true;
+  // the points of the CTA's first tile stay in registers over the steps
+  const int64_t p0 = (int64_t)blockIdx.x * kTT + pl;
+  const float x0 = p0 < A.npts ? A.xy[2 * p0] : 0.f, y0 = p0 < A.npts ? A.xy[2 * p0 + 1] : 0.f;
+  const float tg0 = p0 < A.npts ? A.tgt[p0] : 0.f;
+  for (;; ++t) {
   const bool grad_pass = !ADAM || t < A.steps;
   if (!ADAM || t == 0) {
     // theta as given; launch 0 of a training run also keeps a copy
@@ -158,8 +197,8 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
   } else if (grad_pass || blockIdx.x == 0) {
     // Adam update t from the parameters, moments and gradient of launch t - 1
     const int rd = ((t - 1) & 1) * kMlpParams, wr = (t & 1) * kMlpParams;
-    const float* gp = A.grad + ((t - 1) % 3) * kMlpParams;
-    const float c1 = (float)(1.0 - __ldcg(&A.st->p1)), c2 = (float)(1.0 - __ldcg(&A.st->p2));
+    const float* gp = A.grad + ((t - 1) % 3) * A.grad_stride;
+    const float c1 = (float)(1.0 - p1), c2 = (float)(1.0 - p2);
     // all of a thread's loads in flight at once, then the updates
     float g_[kPer], m_[kPer], v_[kPer], t_[kPer];
 #pragma unroll
@@ -190,34 +229,15 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
       }
     }
   }
-  if (ADAM && blockIdx.x == 0) {
-    // clear the gradient buffer launch t + 1 accumulates into (last read by t - 1)
-    float* gz = A.grad + ((t + 1) % 3) * kMlpParams;
-    for (int i = tid; i < kMlpParams; i += kThreads) gz[i] = 0.f;
+  if (ADAM && grad_pass) {
+    // clear the gradient buffer step t + 1 accumulates into (last read in step t - 1)
+    float* gz = A.grad + ((t + 1) % 3) * A.grad_stride;
+    for (int i = blockIdx.x * kThreads + tid; i < kMlpParams; i += gridDim.x * kThreads) gz[i] = 0.f;
   }
-  // rows 64-79 of the gradient B tile (x, y and 1 are rewritten per tile, the
-  // rest stay zero) and the whole dv tile
-  for (int i = tid; i < 2 * 16 * 128 / 16; i += kThreads) {
-    const int a = i / 128, w = i % 128;  // atom column, 16-byte word within rows 64-79
-    *reinterpret_cast<uint4*>(reinterpret_cast<char*>(S.GB) + a * kBR * 128 + 8 * 1024 + 16 * w) =
-        make_uint4(0u, 0u, 0u, 0u);
-  }
-  for (int i = tid; i < kVR * kTT * 2 / 16; i += kThreads)
-    *reinterpret_cast<uint4*>(reinterpret_cast<char*>(S.DV) + 16 * i) = make_uint4(0u, 0u, 0u, 0u);
-  if (tid == 0) tc::mbar_init(&S.mbar);
-  if (warp == 0) tc::tmem_alloc(&S.tmem, kTmemCols);
   tc::fence_async_smem();
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
-  // warpgroup g takes hidden units [32 g, 32 g + 32) of every point; thread
-  // pl of the group owns point pl of the tile and TMEM lane pl
-  const int g = tid / kTT, pl = tid % kTT;
-  const unsigned tm = S.tmem, tl = (unsigned)((warp & 3) * 32) << 16;
-  const unsigned sP = tc::smem_addr(S.P), sGA = tc::smem_addr(S.GA), sGB = tc::smem_addr(S.GB);
-  const unsigned sDV = tc::smem_addr(S.DV);
-  unsigned phase = 0;
-  bool ok = true;
   float gb3 = 0.f;
   double lsum = 0.0;
   int done = 0;  // tiles this CTA has taken
@@ -225,8 +245,12 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t p = tile * kTT + pl;
     const bool valid = p < A.npts;
-    const float x = valid ? A.xy[2 * p] : 0.f, y = valid ? A.xy[2 * p + 1] : 0.f;
-    const float tg = valid ? A.tgt[p] : 0.f;
+    float x = x0, y = y0, tg = tg0;
+    if (done > 0) {
+      x = valid ? A.xy[2 * p] : 0.f;
+      y = valid ? A.xy[2 * p + 1] : 0.f;
+      tg = valid ? A.tgt[p] : 0.f;
+    }
     // ---- layer 1: h1 into P (row pl) and h1^T (column pl), SiLU'(a1) into TMEM
 #pragma unroll
     for (int qq = 0; qq < 2; ++qq) {
@@ -364,7 +388,8 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
   if (done > 0) {
     // ---- the CTA's partial gradient: TMEM lane pl holds accumulator row pl;
     // the two groups split the columns
-    float* gacc = A.grad + (ADAM ? (t % 3) * kMlpParams : 0);
+    float* gacc = A.grad + (ADAM ? (t % 3) * A.grad_stride : 0);
+    const bool vec = (reinterpret_cast<uintptr_t>(gacc) & 15) == 0;  // (a caller's buffer may not be)
     float gv[16];
     if ((warp & 3) < 2) {  // rows 0-63: output unit o = pl
       const int o = pl;
@@ -372,8 +397,15 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
       for (int qq = 0; qq < 2; ++qq) {
         const int q = 2 * g + qq;
         tc::tmem_ld16(tm + tl + kColG + 16 * q, gv);
+        float* to = gacc + kOffW2 + o * kHU + 16 * q;
+        if (vec) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) atomicAdd(gacc + kOffW2 + o * kHU + 16 * q + j, gv[j]);
+          for (int j = 0; j < 16; j += 4)
+            atomicAdd(reinterpret_cast<float4*>(to + j), make_float4(gv[j], gv[j + 1], gv[j + 2], gv[j + 3]));
+        } else {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) atomicAdd(to + j, gv[j]);
+        }
       }
       if (g == 0) {
         tc::tmem_ld16(tm + tl + kColG + 64, gv);
@@ -409,7 +441,9 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
     }
   }
   if (!ok && tid == 0) atomicAdd(A.loss + t, __longlong_as_double(0x7ff8000000000000ll));
-  if constexpr (ADAM) {
+  if constexpr (!ADAM) {
+    break;
+  } else if (!A.persistent) {
     // the last CTA to arrive advances the step (as in the FP32 kernel)
     if (tid == 0 && atomicAdd(&A.st->count, 1u) == gridDim.x - 1) {
       A.st->count = 0;
@@ -417,6 +451,39 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
       A.st->p2 = (t == 0 ? 1.0 : A.st->p2) * (double)A.beta2;
       A.st->t = t + 1;
     }
+    break;
+  } else {
+    if (!grad_pass) break;
+    p1 *= (double)A.beta1;
+    p2 *= (double)A.beta2;
+    // every CTA's gradient (and CTA 0's parameters) before anyone's next step
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      atomicAdd(&A.st->count, 1u);
+      const unsigned want = (unsigned)(t + 1) * gridDim.x;
+      uint64_t began = 0;
+      bool met = true;
+      for (int spin = 1;; ++spin) {
+        unsigned seen;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&A.st->count) : "memory");
+        if ((int)(seen - want) >= 0) break;
+        if ((spin & 255) == 0) {
+          const uint64_t now = tc::now_ns();
+          if (began == 0) began = now;
+          if (now - began > kWaitNs) { met = false; break; }
+        }
+      }
+      __threadfence();
+      S.met = met ? 1 : 0;
+    }
+    __syncthreads();
+    if (!S.met) {  // a CTA is gone: every later loss is void
+      if (tid == 0)
+        for (int q = t + 1; q < A.steps; ++q) atomicAdd(A.loss + q, __longlong_as_double(0x7ff8000000000000ll));
+      break;
+    }
+  }
   }
   tc::fence_before();
   __syncthreads();
