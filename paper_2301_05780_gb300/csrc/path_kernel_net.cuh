@@ -291,8 +291,8 @@ __global__ void __launch_bounds__(kNetRows, 5)
   if (tid == 0) {
     s_live = 0;
     s_qempty = 0;
-    for (int s = 0; s < 2; ++s) {
-      S.st(s).ctrl = (unsigned long long)(2u * s + 1u) << 32;  // "loading unit s"
+    for (int s = 0; s < P.stages; ++s) {
+      S.st(s).ctrl = 1ull << 32;  // "loading its unit 0"
       S.st(s).term = 0;
       S.st(s).tma_phase = 0;
       mbar_init(&S.st(s).mbar);
@@ -308,7 +308,8 @@ __global__ void __launch_bounds__(kNetRows, 5)
   __syncthreads();
   tc::fence_after();
   bool ok = true;
-  if (warp < 2) ok = load_unit<EXT>(S, warp, warp, P, total_units, units_done);
+  for (int s = warp; s < P.stages && ok; s += kNetRows / 32)
+    ok = load_unit<EXT>(S, s, 0, P, total_units, units_done);
   __syncthreads();
   const unsigned tm = N.tmem, ts = N.tmem_s1;
   const unsigned tl = (unsigned)((warp & 3) * 32) << 16;
@@ -322,7 +323,7 @@ __global__ void __launch_bounds__(kNetRows, 5)
   float xk = 0.f, yk = 0.f, bx0 = 0.f, bx1 = 0.f, by0 = 0.f, by1 = 0.f;
   float X = 0.f, Y = 0.f, Sx = 0.f, Z = 0.f, XI = 0.f;
   unsigned long long my_steps = 0, my_paths = 0, my_trunc = 0, my_clamp = 0;
-  int want = 0;
+  int from = warp % P.stages;
   // EXT: the knot's step, its square root, step cap and Gobet-Menozzi shift
   // per unit of |s|; the mixed GM/EM run of the calibration (records kernels
   // with the extended exit) as in path_kernel
@@ -343,11 +344,17 @@ __global__ void __launch_bounds__(kNetRows, 5)
     // ---- hand new paths to idle lanes (per warp, never waits) --------------
     unsigned idle = __ballot_sync(kFull, !alive);
     for (int guard = 0; idle && guard < 64; ++guard) {
-      Stage& H = S.st(want & 1);
-      const unsigned ss = ctrl_state(&H.ctrl);
-      if ((int)(ss >> 1) > want) { ++want; continue; }
-      if ((ss & 1u) || (int)(ss >> 1) < want) break;
-      if (H.term) { ++want; continue; }
+      bool has = false;  // lane s: stage s published, with paths left? (as in path_kernel)
+      if (lane < P.stages) {
+        Stage& Q = S.st(lane);
+        const unsigned long long v = ctrl_word(&Q.ctrl);
+        has = !((v >> 32) & 1ull) && !Q.term && (int)(unsigned)v < Q.p_end;
+      }
+      const unsigned avail = __ballot_sync(kFull, has);
+      if (avail == 0) break;
+      const unsigned ahead = avail >> from << from;
+      from = __ffs(ahead ? ahead : avail) - 1;
+      Stage& H = S.st(from);
       const int cnt = __popc(idle);
       const int leader = __ffs(idle) - 1;
       unsigned long long c = 0;
@@ -355,20 +362,16 @@ __global__ void __launch_bounds__(kNetRows, 5)
       c = __shfl_sync(kFull, c, leader);
       __threadfence_block();
       const unsigned sa = (unsigned)(c >> 32);
-      if (sa & 1u) break;
+      if (sa & 1u) continue;
       const int base = (int)(unsigned)(c & 0xffffffffull);
       const int pend = H.p_end;
       __threadfence_block();
-      if (ctrl_state(&H.ctrl) != sa) {
-        want = max(want, (int)(sa >> 1) + 1);
-        continue;
-      }
-      want = max(want, (int)(sa >> 1));
+      if (ctrl_state(&H.ctrl) != sa) continue;
       const int got = max(0, min(cnt, pend - base));
       const int rank = __popc(idle & ((1u << lane) - 1u));
       if (!alive && rank < got) {
         alive = true;
-        st = want & 1;
+        st = from;
         p = (uint32_t)(base + rank);
         kk = (uint32_t)H.k;
         tagw = (uint32_t)H.tag;
@@ -386,7 +389,6 @@ __global__ void __launch_bounds__(kNetRows, 5)
         }
         n = 0; X = 0.f; Y = 0.f; Sx = 0.f; Z = 0.f; XI = 0.f;
       }
-      if (base + cnt >= pend) ++want;
       idle = __ballot_sync(kFull, !alive);
     }
     if (!group_any(g, alive)) {
@@ -545,11 +547,10 @@ __global__ void __launch_bounds__(kNetRows, 5)
     }
     // warp-aggregated completion counts per stage; the warp that finishes a
     // unit flushes it and loads the next one (bounded waits only)
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const unsigned m = __ballot_sync(kFull, leaving && !gm_rec && st == s);
-      if (m == 0) continue;
-      __syncwarp();
+    for (unsigned gone = __ballot_sync(kFull, leaving && !gm_rec); gone != 0;) {
+      const int s = __shfl_sync(kFull, st, __ffs(gone) - 1);
+      const unsigned m = __ballot_sync(kFull, st == s) & gone;
+      gone &= ~m;
       __threadfence_block();
       int fin = 0;
       if (lane == 0) {
@@ -561,7 +562,7 @@ __global__ void __launch_bounds__(kNetRows, 5)
       if (fin) {
         const int q = (int)(ctrl_state(&S.st(s).ctrl) >> 1);
         flush_unit(S, s, P);
-        if (!load_unit<EXT>(S, s, q + 2, P, total_units, units_done)) ok = false;
+        if (!load_unit<EXT>(S, s, q + 1, P, total_units, units_done)) ok = false;
         if (lane == 0) atomicSub(S.live, 1);
         __syncwarp();
       }

@@ -427,12 +427,12 @@ int64_t default_kmax(const pdds_ctx* c, double dt) {
   return (int64_t)std::ceil(40.0 * T / dt);
 }
 
-// The shape of one path-kernel launch.
+// The shape of one path-kernel launch (units: at least so many it will have).
 struct LaunchPlan {
   int cv = 0, block = 0, grid = 0, exit_batch = 0, stages = 2;
   size_t smem = 0;
   int64_t unit_paths = 0;  // 0: auto_unit_paths
-  int64_t warps() const { return block / 32; }
+  pdds::UnitRule rule() const { return {grid, block / 32, cv == 3 ? 1 : 0}; }
 };
 
 // Fields that pdds_set_launch or pdds_autotune have set are kept; the others:
@@ -445,7 +445,7 @@ struct LaunchPlan {
 //  - exit batch: 4 lanes, 8 where a path takes fewer steps than two visits of
 //    the step loop (2 % on paths of 11 steps, 2-4 % slower on long ones).
 pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob, size_t sbytes,
-                        double dt, LaunchPlan& L) {
+                        double dt, int64_t units, LaunchPlan& L) {
   // cv 3: the in-path network on tcgen05 (the warpgroup kernel)
   L.cv = nprob == 1 ? c->cv_mode : 0;
   if (L.cv == 1 && c->net_engine == PDDS_NET_TCGEN05) L.cv = 3;
@@ -480,29 +480,31 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
   }
   // tcgen05 kernel: 96 TMEM columns per CTA, 512 per SM
   if (L.cv == 3) per_sm = std::min(per_sm, 512 / 96);
-  if (L.cv != 3) {
-    // A unit's stage is free again only when its last path has left, so with
-    // two stages the lanes run dry where units are short (per-knot budgets,
-    // wide stencils): a third one, where the resident CTAs stay and, with the
-    // tabulated control variate, the L1 cache keeps 60 KB for the table.  One
-    // GB300, two / three / four stages: RBF stencils 9.6 / 8.9 / 8.9 ms, the
-    // paper's production run 45.3 / 42.1 / 43.1, batch of 16 461 / 455 / 455;
-    // L1 below 50 KB: 56.
-    const size_t three = 3 * sbytes + net;
-    if (three * per_sm <= (L.cv == 2 ? 160 : 227) * 1024) {
-      int ctas = 0;
-      CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, three));
-      CK(c, pdds::path_kernel_occupancy(coef_id, rec, L.cv, ext, L.block, three, &ctas));
-      if (ctas >= per_sm) {
-        L.stages = 3;
-        L.smem = three;
-      }
+  // A unit's stage is free again only when its last path has left, so with two
+  // stages the lanes run dry where units are short (per-knot budgets, wide
+  // stencils, 128 lanes of the warpgroup kernel on 11-step paths).  More of
+  // them, where the resident CTAs stay, every CTA still gets as many units (a
+  // knot has at least one) and, with the tabulated control variate, the L1
+  // cache keeps 60 KB for the table.  One GB300, two / three / four stages: RBF
+  // stencils 9.6 / 8.9 / 8.9 ms, the paper's production run 45.3 / 42.1 / 43.1
+  // (L1 below 50 KB: 56), batch of 16 461 / 455 / 455; in-path network on 11-step
+  // paths, 100 per knot, two / three / four / eight: 17.1 / 12.4 / 10.1 / 8.0.
+  for (int r = L.cv == 3 ? 8 : 3; r > 2; --r) {
+    const size_t smem = r * sbytes + net;
+    const int64_t ctas_all = (int64_t)c->num_sms * per_sm;
+    if (units < r * ctas_all || smem * per_sm > (size_t)(L.cv == 2 ? 160 : 227) * 1024) continue;
+    int ctas = 0;
+    CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, smem));
+    CK(c, pdds::path_kernel_occupancy(coef_id, rec, L.cv, ext, L.block, smem, &ctas));
+    if (ctas >= per_sm) {
+      L.stages = r;
+      L.smem = smem;
+      break;
     }
-    CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, L.smem));
   }
+  CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, L.smem));
   L.grid = c->num_sms * per_sm;
-  // (the warpgroup kernel steps 128 paths at a time, however few are left)
-  L.unit_paths = c->auto_unit && L.cv != 3 ? 0 : c->unit_paths;
+  L.unit_paths = c->auto_unit ? 0 : c->unit_paths;
   L.exit_batch = !c->auto_batch ? c->exit_batch : mean_steps_estimate(c, dt) < 32.0 ? 8 : 4;
   return PDDS_OK;
 }
@@ -600,21 +602,21 @@ pdds_status assemble_impl(pdds_ctx* c, const int64_t* N, int64_t Nu, double dt, 
   const bool gm = (scheme < 0 ? c->scheme : scheme) == PDDS_SCHEME_GM;
   const bool ext = gm || c->d_hknot != nullptr || c->interp == PDDS_INTERP_RBF;
   LaunchPlan L;
-  if (pdds_status e = plan_launch(c, c->coef_id, rec != nullptr, ext, 1, stage_bytes(c), dt, L)) return e;
+  if (pdds_status e = plan_launch(c, c->coef_id, rec != nullptr, ext, 1, stage_bytes(c), dt, c->geo.n, L)) return e;
   ProbDesc D = make_prob(c, (int)c->tag);
   D.Gval = G->val;
   D.b = b;
   D.n_per_knot = N;
   D.n_paths = Nu;
   if (N) {
-    CK(c, pdds::launch_unit_prefix(N, c->geo.n, L.unit_paths, 1, L.grid, L.warps(), c->d_unit_prefix,
+    CK(c, pdds::launch_unit_prefix(N, c->geo.n, L.unit_paths, 1, L.rule(), c->d_unit_prefix,
                                    c->d_path_prefix, &c->d_scratch->error, s));
     ++launches;
     D.knot_unit_prefix = c->d_unit_prefix;
     D.path_prefix = c->d_path_prefix;
   } else {
     D.unit_paths = L.unit_paths ? L.unit_paths
-                                : pdds::auto_unit_paths(c->geo.n * Nu, L.grid, L.warps());
+                                : pdds::auto_unit_paths(c->geo.n * Nu, L.rule());
     D.units_per_knot = ceil_div(Nu, D.unit_paths);
   }
   CK(c, pdds::launch_prob_prefix_single(D, c->d_prob_prefix, s));
@@ -1386,7 +1388,7 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
   (void)cudaGetLastError();
   if (!(dt > 0)) return fail(c0, PDDS_EINVAL, "assemble_batch: dt must be > 0");
   int max_slots = 0, tw = 0, th = 0;
-  int64_t kmax = 0;
+  int64_t kmax = 0, knots = 0;
   double dom_bound = 0.0;  // max |coordinate| over the batch's domains
   for (int i = 0; i < count; ++i) {
     pdds_ctx* c = ctxs[i];
@@ -1406,6 +1408,7 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
     if (pdds_status e = check_csr(c, G[i], b[i])) return fail(c0, e, c->err);
     if (!(N && N[i]) && (Nu < 1 || Nu >= ((int64_t)1 << 31)))
       return fail(c0, PDDS_EINVAL, "assemble_batch: n_paths must be in [1, 2^31)");
+    knots += c->geo.n;
     max_slots = std::max(max_slots, c->geo.max_slots);
     tw = std::max(tw, c->tile_w);
     th = std::max(th, c->tile_h);
@@ -1437,7 +1440,7 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
       return round_up(x, 128);
     }();
     LaunchPlan L;
-    if (pdds_status e = plan_launch(c0, c0->coef_id, false, false, count == 1 ? 1 : 2, sb, dt, L))
+    if (pdds_status e = plan_launch(c0, c0->coef_id, false, false, count == 1 ? 1 : 2, sb, dt, knots, L))
       return e;
     std::vector<ProbDesc> probs(count);
     for (int i = 0; i < count; ++i) {
@@ -1453,7 +1456,7 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
       } else {
         // the launch's paths are about `count` times this problem's
         D.unit_paths = L.unit_paths ? L.unit_paths
-                                    : pdds::auto_unit_paths(count * c->geo.n * Nu, L.grid, L.warps());
+                                    : pdds::auto_unit_paths(count * c->geo.n * Nu, L.rule());
         D.units_per_knot = ceil_div(Nu, D.unit_paths);
       }
       probs[i] = D;
@@ -1495,7 +1498,7 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
     for (int i = 0; N && i < count; ++i) {
       pdds_ctx* c = ctxs[i];
       if (N[i])
-        step(pdds::launch_unit_prefix(N[i], c->geo.n, L.unit_paths, count, L.grid, L.warps(),
+        step(pdds::launch_unit_prefix(N[i], c->geo.n, L.unit_paths, count, L.rule(),
                                       c->d_unit_prefix, c->d_path_prefix, &c0->d_scratch->error, s),
              "unit prefix");
     }

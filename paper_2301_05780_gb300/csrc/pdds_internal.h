@@ -141,22 +141,27 @@ cudaError_t mlp_stage(const float* theta, void* image, cudaStream_t stream);
 //    2.9e5 paths 2.2 -> 0.6 ms; 1.3e6 1.6 -> 0.75; 1.2e6 variable-sigma paths
 //    7.6 -> 5.3; from 5e6 paths on the upper end is within 1 % of the best);
 //  - fewer paths than lanes: one unit per warp, so that every warp has as few
-//    paths as possible (its idle lanes then draw ahead for them).
-__host__ __device__ inline int64_t auto_unit_paths(int64_t paths, int64_t ctas, int64_t warps) {
-  if (paths <= ctas * warps * 32) {
-    const int64_t u = (paths + ctas * warps - 1) / (ctas * warps);
+//    paths as possible (its idle lanes then draw ahead for them); not for the
+//    warpgroup kernel (whole_ctas), which steps 128 paths at a time.
+struct UnitRule {
+  int64_t ctas, warps;
+  int32_t whole_ctas;
+};
+__host__ __device__ inline int64_t auto_unit_paths(int64_t paths, const UnitRule& r) {
+  const int64_t lo = 32 * r.warps, hi = 256 * r.warps;
+  if (!r.whole_ctas && paths <= r.ctas * lo) {
+    const int64_t u = (paths + r.ctas * r.warps - 1) / (r.ctas * r.warps);
     return u < 1 ? 1 : u;
   }
-  const int64_t u = paths * 2 / (5 * ctas), lo = 32 * warps, hi = 256 * warps;
+  const int64_t u = paths * 2 / (5 * r.ctas);
   return u < lo ? lo : u > hi ? hi : u;
 }
 // Unit and record prefixes of per-knot budgets; unit_paths 0: auto_unit_paths
 // of `share` times the knots' paths (share: problems of the launch).
 // Budgets outside [0, 2^31) count as zero paths and set *err = PDDS_EINVAL.
 cudaError_t launch_unit_prefix(const int64_t* n_per_knot, int64_t n, int64_t unit_paths,
-                               int64_t share, int64_t ctas, int64_t warps,
-                               int64_t* knot_unit_prefix, int64_t* path_prefix, int32_t* err,
-                               cudaStream_t stream);
+                               int64_t share, const UnitRule& rule, int64_t* knot_unit_prefix,
+                               int64_t* path_prefix, int32_t* err, cudaStream_t stream);
 cudaError_t launch_cv_cells(const float* nodes, int nx, int ny, float* cells, cudaStream_t s);
 cudaError_t launch_prob_prefix_single(const ProbDesc& D, int64_t* out, cudaStream_t stream);
 cudaError_t launch_prob_prefix(const ProbDesc* probs, int nprob, int64_t* out, cudaStream_t stream);

@@ -27,7 +27,7 @@ __device__ __forceinline__ int64_t checked_budget(int64_t v, bool& bad) {
 // PDDS_EINVAL in *err.  The records' prefix comes first: its total decides the
 // unit size when the caller has set none (C == 0).
 __global__ void unit_prefix_kernel(const int64_t* __restrict__ N, int64_t n, int64_t C, int64_t share,
-                                   int64_t ctas, int64_t warps, int64_t* __restrict__ up,
+                                   const UnitRule rule, int64_t* __restrict__ up,
                                    int64_t* __restrict__ pp, int32_t* __restrict__ err) {
   __shared__ int64_t sum[1024];
   const int t = threadIdx.x, T = blockDim.x;
@@ -56,7 +56,7 @@ __global__ void unit_prefix_kernel(const int64_t* __restrict__ N, int64_t n, int
     before += checked_budget(N[i], bad);
   }
   const int64_t total = sum[T - 1];
-  if (C == 0) C = auto_unit_paths(share * total, ctas, warps);
+  if (C == 0) C = auto_unit_paths(share * total, rule);
   v = 0;
   for (int64_t i = lo; i < hi; ++i) v += (checked_budget(N[i], bad) + C - 1) / C;
   before = scan(v);
@@ -172,10 +172,10 @@ cudaError_t set_path_kernel_smem(int coef, bool rec, int cv, bool ext, size_t sm
   return e;
 }
 
-cudaError_t launch_unit_prefix(const int64_t* N, int64_t n, int64_t C, int64_t share, int64_t ctas,
-                               int64_t warps, int64_t* up, int64_t* pp, int32_t* err,
+cudaError_t launch_unit_prefix(const int64_t* N, int64_t n, int64_t C, int64_t share,
+                               const UnitRule& rule, int64_t* up, int64_t* pp, int32_t* err,
                                cudaStream_t stream) {
-  unit_prefix_kernel<<<1, 1024, 0, stream>>>(N, n, C, share, ctas, warps, up, pp, err);
+  unit_prefix_kernel<<<1, 1024, 0, stream>>>(N, n, C, share, rule, up, pp, err);
   return cudaGetLastError();
 }
 
