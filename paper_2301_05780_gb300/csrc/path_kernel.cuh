@@ -269,9 +269,22 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
 }
 
 // ----------------------------------------------------------- coefficients
+// The hardware reciprocal and reciprocal square root without the scaling that
+// their default forms add for denormal arguments and results (a few
+// instructions each); used where neither occurs, so the values are the same.
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 // tanh q = 1 - 2 / (e^{2q} + 1) (|q| <= 2 for the problem below).
 __device__ __forceinline__ float tanh_small(float q) {
-  return 1.0f - __fdividef(2.0f, __expf(2.0f * q) + 1.0f);
+  return fmaf(-2.0f, rcp_approx(ex2_approx((2.0f * q) * 1.44269504088896341f) + 1.0f), 1.0f);
 }
 
 // The Poisson problem of Sec. 5.1 (Eq. 42-43): u = 3 + sin(r)/3 + tanh(q)/3 with
@@ -295,8 +308,9 @@ __device__ __forceinline__ void sincos_rad(float a, bool direct, float& s, float
 __device__ __forceinline__ E1Terms e1_terms(float x, float y, float r, bool direct) {
   E1Terms t;
   sincos_rad(r, direct, t.sr, t.cr);
-  sincos_rad(fmaf(0.12f, x, 0.05f * y), direct, t.sa, t.ca);
-  sincos_rad(fmaf(0.05f, x, -0.12f * y), direct, t.sb, t.cb);
+  const float2 ab = fma2(f2(0.12f, 0.05f), f2(x, x), mul2(f2(0.05f, -0.12f), f2(y, y)));
+  sincos_rad(ab.x, direct, t.sa, t.ca);
+  sincos_rad(ab.y, direct, t.sb, t.cb);
   t.q = t.sa + t.sb;
   t.T = tanh_small(t.q);
   return t;
@@ -313,13 +327,13 @@ __device__ __forceinline__ float e1_u(float x, float y) {
 // (r^2 >= 1; a few ulp, far below the FP32 path rounding), r = r^2 / r.
 __device__ __forceinline__ float e1_lap(float x, float y, bool direct) {
   const float r2 = e1_r2(x, y);
-  const float ir = rsqrtf(r2);
+  const float ir = rsqrt_approx(r2);
   const E1Terms t = e1_terms(x, y, r2 * ir, direct);
   const float Gi2 = fmaf(x * x, 1e-4f, y * y * 4e-4f) * (ir * ir);  // G / r^2
   const float lap_r = ir * (0.03f - Gi2);                           // 0.03 / r - G / r^3
   const float lap_sin = fmaf(t.cr, lap_r, -t.sr * Gi2);
-  const float qx = fmaf(0.12f, t.ca, 0.05f * t.cb);
-  const float qy = fmaf(0.05f, t.ca, -0.12f * t.cb);
+  const float2 dq = fma2(f2(0.12f, 0.05f), f2(t.ca, t.ca), mul2(f2(0.05f, -0.12f), f2(t.cb, t.cb)));
+  const float qx = dq.x, qy = dq.y;
   const float lap_q = -0.0169f * t.q;
   const float lap_tanh = (1.0f - t.T * t.T) * fmaf(-2.0f * t.T, fmaf(qx, qx, qy * qy), lap_q);
   return (lap_sin + lap_tanh) * 0.333333343f;
@@ -416,11 +430,13 @@ __device__ __forceinline__ void coeffs(const Stage& H, const float* tsig, const 
     // s = sqrt2 (1 + 0.3 sin 2 pi x sin 2 pi y), c = -1, u = e^{x/4} cos(y/2),
     // f = (s^2/2)(1/16 - 1/4) u + c u.
     float s1, c1, s2, c2, sh, ch;
+    // the exponent of u and half of y as one packed product
+    const float2 e = mul2(f2(0.360673760222241f, 0.5f), f2(x, y));
     if (trig_direct) {  // |x|, |y| <= 7 (set on the host): angles below 45 rad
       const float2 a = mul2(f2(kTwoPi, kTwoPi), f2(x, y));
       s1 = __sinf(a.x);
       s2 = __sinf(a.y);
-      ch = __cosf(0.5f * y);
+      ch = __cosf(e.y);
       (void)c1; (void)c2; (void)sh;
     } else {
       sincos_2pi(x, s1, c1);
@@ -429,10 +445,11 @@ __device__ __forceinline__ void coeffs(const Stage& H, const float* tsig, const 
     }
     // q = s / sqrt2; u = 2^{x log2(e) / 4} cos(y/2); f = -u (1 + (3/16) q^2)
     const float q = fmaf(0.3f * s1, s2, 1.0f);
-    s = 1.41421356237309505f * q;
-    const float u = ex2_approx(x * 0.360673760222241f) * ch;
+    const float2 sq = mul2(f2(1.41421356237309505f, 0.1875f), f2(q, q));
+    s = sq.x;
+    const float u = ex2_approx(e.x) * ch;
     dx = 0.f; dy = 0.f; c = -1.0f;
-    f = -u * fmaf(0.1875f * q, q, 1.0f);
+    f = -u * fmaf(sq.y, q, 1.0f);
   } else if constexpr (COEF == PDDS_COEF_TABLE) {
     const float fx = fmaf(xr, H.tab_inv_dx, H.kd.tab_fx);
     const float fy = fmaf(yr, H.tab_inv_dy, H.kd.tab_fy);
@@ -512,24 +529,28 @@ __device__ __forceinline__ const ProbDesc& prob_desc(const KParams& P, int i) {
 
 // Tabulated control variate (Sec. 4.2): grad u0 at the [cv_ny][cv_nx] nodes
 // spanning Omega, bilinear in between, kept cell by cell: cell (i, j) holds
-// its four corners' gx then gy (32 bytes, one sector; read through L1/L2),
-// one lookup = two 16-byte loads of one sector instead of four 8-byte loads
-// from two rows (7 % faster per step on the paper's problem).
+// its four corners (gx, gy) in node order (32 bytes, one sector; read through
+// L1/L2), one lookup = two 16-byte loads of one sector instead of four 8-byte
+// loads from two rows (7 % faster per step on the paper's problem).  Both
+// components are interpolated at once in packed FP32 (six instructions instead
+// of twelve), and the weights are clamped by the subtraction's saturation.
 __device__ __forceinline__ void cv_table_grad(const ProbDesc& D, float x, float y, float& gx,
                                               float& gy) {
   const float fx = (x - D.x0) * D.cv_inv_dx, fy = (y - D.y0) * D.cv_inv_dy;
   const int i = min(max((int)floorf(fx), 0), D.cv_nx - 2);
   const int j = min(max((int)floorf(fy), 0), D.cv_ny - 2);
-  const float tx = fminf(fmaxf(fx - (float)i, 0.f), 1.f);
-  const float ty = fminf(fmaxf(fy - (float)j, 0.f), 1.f);
-  // cell-major table: the four corners of cell (i, j), gx then gy, in one sector
-  const float4* cell = reinterpret_cast<const float4*>(D.cv_tab) +
-                       2 * ((int64_t)j * (D.cv_nx - 1) + i);
+  const float tx = __saturatef(fx - (float)i);
+  const float ty = __saturatef(fy - (float)j);
+  // (at most 2^28 nodes: the cell index fits 32 bits)
+  const float4* cell = reinterpret_cast<const float4*>(D.cv_tab) + 2 * (int64_t)(j * (D.cv_nx - 1) + i);
   const float4 G = __ldg(cell), H = __ldg(cell + 1);
-  const float x0 = fmaf(tx, G.y - G.x, G.x), x1 = fmaf(tx, G.w - G.z, G.z);
-  const float y0 = fmaf(tx, H.y - H.x, H.x), y1 = fmaf(tx, H.w - H.z, H.z);
-  gx = fmaf(ty, x1 - x0, x0);
-  gy = fmaf(ty, y1 - y0, y0);
+  const float2 n00 = f2(G.x, G.y), n01 = f2(G.z, G.w), n10 = f2(H.x, H.y), n11 = f2(H.z, H.w);
+  const float2 m1 = f2(-1.0f, -1.0f);
+  const float2 b = fma2(f2(tx, tx), fma2(n00, m1, n01), n00);
+  const float2 t = fma2(f2(tx, tx), fma2(n10, m1, n11), n10);
+  const float2 g = fma2(f2(ty, ty), fma2(b, m1, t), b);
+  gx = g.x;
+  gy = g.y;
 }
 
 // One Euler-Maruyama step (Eq. 9, Sec. 2.3) of a lane's path, in place:

@@ -199,8 +199,8 @@ __global__ void cv_cells_kernel(const float* __restrict__ nodes, int nx, int ny,
   const float2 a = n2[(int64_t)j * nx + i], b = n2[(int64_t)j * nx + i + 1];
   const float2 d0 = n2[(int64_t)(j + 1) * nx + i], d1 = n2[(int64_t)(j + 1) * nx + i + 1];
   float4* o = reinterpret_cast<float4*>(cells) + 2 * c;
-  o[0] = make_float4(a.x, b.x, d0.x, d1.x);
-  o[1] = make_float4(a.y, b.y, d0.y, d1.y);
+  o[0] = make_float4(a.x, a.y, b.x, b.y);
+  o[1] = make_float4(d0.x, d0.y, d1.x, d1.y);
 }
 
 cudaError_t launch_cv_cells(const float* nodes, int nx, int ny, float* cells, cudaStream_t s) {
