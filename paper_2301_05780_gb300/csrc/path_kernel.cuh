@@ -750,6 +750,17 @@ __device__ __forceinline__ void coop_calls(const PathConst& c, const KParams& P,
   }
 }
 
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+  return v;
+}
+__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+  return v;
+}
+
 // What the resolution of one exited path produces (Eq. 22-25).
 struct ExitResult {
   double bc = 0.0;          // the path's share of b_k (times N_k)
@@ -878,6 +889,58 @@ __device__ __forceinline__ ExitResult resolve_exit(const Smem& S, const KParams&
     }
   }
   return E;
+}
+
+// An RBF interface exit at coordinate sl of the stencil of side `side`, by the
+// whole warp: knot j of the stencil gets Y H_j(sl) (deposit: into the slot
+// accumulators), the stencil's knots on the boundary of Omega add Y H_j g(x_j)
+// to the returned sum (the path's share of b).  A lane evaluates K of its knots'
+// Chebyshev series side by side: a recurrence is a serial chain of one table
+// load and one FMA per coefficient, so a warp that takes a 145-knot stencil's
+// five per lane one after the other waits five times as long.  One GB300, the
+// paper's problem at 200 paths per knot: K = 1 / 2 / 3 / 5 8.9 / 7.3 / 6.9 / 6.6 ms;
+// three, since five cost the same kernel's step loop registers (variable sigma
+// 4 % slower).  The records kernels, whose loop has none to spare (calibration
+// 2.4 % slower with three), keep one.
+template <int COEF, int K>
+__device__ __forceinline__ double rbf_deposit(const Stage& H, unsigned long long* acc, const ProbDesc& D,
+                                              int side, float sl, float Y, bool deposit,
+                                              int32_t* error) {
+  const int lane = threadIdx.x & 31;
+  const KnotDesc& kd = H.kd;
+  const bool vertical = (side == 0 || side == 2);
+  const int a = kd.a[side];
+  const int L = kd.b[side] - a + 1;
+  const int lmax = vertical ? H.LY : H.LX;
+  float tau;
+  const float* cf = rbf_interval(D, vertical ? 1 : 0, L, sl, tau);
+  double dsum = 0.0;
+  if (cf == nullptr) {
+    if (lane == 0) atomicExch(error, (int)PDDS_EINVAL);
+    return 0.0;
+  }
+  const int P1 = D.rbf_deg + 1;
+  for (int j0 = lane; j0 < L; j0 += 32 * K) {
+    float w[K];
+    rbf_cardinals<K>(cf, L, P1, j0, tau, w);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int j = j0 + 32 * k;
+      if (j >= L) break;
+      const float wj = Y * w[k];
+      const int tl = a + j;
+      if (tl == 0 || tl == lmax) {
+        const int li = vertical ? kd.line[side] : tl;
+        const int lj = vertical ? tl : kd.line[side];
+        dsum += (double)wj * (double)g_value<COEF>(H, fmaf((float)li, H.dx, H.x0),
+                                                   fmaf((float)lj, H.dy, H.y0));
+      } else if (deposit) {
+        // signed weights in 2^-30 units (two's complement in the slot)
+        atomicAdd(acc + kd.off[side] + j, (unsigned long long)__float2ll_rn(wj * kFixedOne));
+      }
+    }
+  }
+  return warp_sum(dsum);
 }
 
 // The per-path record of a resolved exit (knot-major: the record prefix of
@@ -1057,17 +1120,6 @@ __device__ void flush_unit(const Smem& S, int s, const KParams& P) {
   }
   if (lane == 0) atomicAdd(D.b + H.k, H.bsum);
   __syncwarp();
-}
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  return v;
-}
-__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  return v;
 }
 
 // ------------------------------------------------------------- the kernel
@@ -1331,33 +1383,8 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
         const float r_Y = __shfl_sync(kFull, Yk, src);
         bool r_gm = false;
         if constexpr (kMixed) r_gm = __shfl_sync(kFull, gm_rec ? 1 : 0, src) != 0;
-        const Stage& H = S.st(r_st);
-        const KnotDesc& kd = H.kd;
-        const ProbDesc& D = prob_desc(P, H.prob);
-        const bool vertical = (r_side == 0 || r_side == 2);
-        const int a = kd.a[r_side];
-        const int L = kd.b[r_side] - a + 1;
-        const int lmax = vertical ? H.LY : H.LX;
-        float tau;
-        const float* cf = rbf_interval(D, vertical ? 1 : 0, L, r_s, tau);
-        unsigned long long* acc = S.acc(r_st);
-        double dsum = 0.0;
-        if (cf == nullptr && lane == 0) atomicExch(&P.scratch->error, (int)PDDS_EINVAL);
-        for (int j = lane; cf != nullptr && j < L; j += 32) {
-          const float w = r_Y * rbf_cardinal(cf, L, D.rbf_deg + 1, j, tau);
-          const int tl = a + j;
-          if (tl == 0 || tl == lmax) {
-            const int li = vertical ? kd.line[r_side] : tl;
-            const int lj = vertical ? tl : kd.line[r_side];
-            dsum += (double)w * (double)g_value<COEF>(H, fmaf((float)li, H.dx, H.x0),
-                                                      fmaf((float)lj, H.dy, H.y0));
-          } else if (!r_gm) {
-            // signed weights in 2^-30 units (two's complement in the slot)
-            atomicAdd(acc + kd.off[r_side] + j,
-                      (unsigned long long)__float2ll_rn(w * kFixedOne));
-          }
-        }
-        dsum = warp_sum(dsum);
+        const double dsum = rbf_deposit<COEF, RECORD ? 1 : 3>(S.st(r_st), S.acc(r_st), P.prob0, r_side, r_s, r_Y, !r_gm,
+                                              &P.scratch->error);
         if (lane == src) bc += dsum;
         pend &= pend - 1;
       }

@@ -491,31 +491,8 @@ __global__ void __launch_bounds__(kNetRows, 5)
         const float r_Y = __shfl_sync(kFull, E.Yk, src);
         bool r_gm = false;
         if constexpr (kMixed) r_gm = __shfl_sync(kFull, gm_rec ? 1 : 0, src) != 0;
-        const Stage& H = S.st(r_st);
-        const KnotDesc& kd = H.kd;
-        const ProbDesc& D = prob_desc(P, H.prob);
-        const bool vertical = (r_side == 0 || r_side == 2);
-        const int a = kd.a[r_side];
-        const int L = kd.b[r_side] - a + 1;
-        const int lmax = vertical ? H.LY : H.LX;
-        float tau;
-        const float* cf = rbf_interval(D, vertical ? 1 : 0, L, r_s, tau);
-        unsigned long long* acc = S.acc(r_st);
-        double dsum = 0.0;
-        if (cf == nullptr && lane == 0) atomicExch(&P.scratch->error, (int)PDDS_EINVAL);
-        for (int j = lane; cf != nullptr && j < L; j += 32) {
-          const float w = r_Y * rbf_cardinal(cf, L, D.rbf_deg + 1, j, tau);
-          const int tl2 = a + j;
-          if (tl2 == 0 || tl2 == lmax) {
-            const int li = vertical ? kd.line[r_side] : tl2;
-            const int lj = vertical ? tl2 : kd.line[r_side];
-            dsum += (double)w * (double)g_value<COEF>(H, fmaf((float)li, H.dx, H.x0),
-                                                      fmaf((float)lj, H.dy, H.y0));
-          } else if (!r_gm) {
-            atomicAdd(acc + kd.off[r_side] + j, (unsigned long long)__float2ll_rn(w * kFixedOne));
-          }
-        }
-        dsum = warp_sum(dsum);
+        const double dsum = rbf_deposit<COEF, 1>(S.st(r_st), S.acc(r_st), P.prob0, r_side, r_s, r_Y, !r_gm,
+                                              &P.scratch->error);
         if (lane == src) E.bc += dsum;
         pend &= pend - 1;
       }

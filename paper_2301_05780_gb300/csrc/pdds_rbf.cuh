@@ -37,4 +37,29 @@ __device__ __forceinline__ float rbf_cardinal(const float* cf, int L, int P1, in
   return fmaf(tau, b1, __ldg(cf + j) - b2);
 }
 
+// H_j for the knots j0, j0 + 32, ... (K of them) of a lane at once:
+// independent recurrences, each exactly rbf_cardinal's, whose loads are in
+// flight together.  Knots past the stencil's end get 0.
+template <int K>
+__device__ __forceinline__ void rbf_cardinals(const float* cf, int L, int P1, int j0, float tau,
+                                              float (&H)[K]) {
+  float b1[K], b2[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) b1[k] = b2[k] = 0.f;
+  const float t2 = 2.0f * tau;
+  const float* c = cf + (int64_t)(P1 - 1) * L + j0;
+#pragma unroll 2
+  for (int n = P1 - 1; n >= 1; --n, c -= L) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const float v = fmaf(t2, b1[k], (j0 + 32 * k < L ? __ldg(c + 32 * k) : 0.f) - b2[k]);
+      b2[k] = b1[k];
+      b1[k] = v;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    H[k] = j0 + 32 * k < L ? fmaf(tau, b1[k], __ldg(c + 32 * k) - b2[k]) : 0.f;
+}
+
 }  // namespace pdds
