@@ -1397,7 +1397,6 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
         my_clamp += (flags >> 1) & 1;
       }
       if constexpr (RECORD) write_record(S, P, st, kk, p, n, E, XI, gm_rec);
-      if (!gm_rec) atomicAdd(&S.st(st).bsum, bc);  // one FP64 shared atomic per exit
     }
     if constexpr (kMixed) {
       if (gm_rec) {
@@ -1419,6 +1418,17 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
       const int s = __shfl_sync(kFull, st, __ffs(gone) - 1);
       const unsigned m = __ballot_sync(kFull, st == s) & gone;
       gone &= ~m;
+      // The exits' shares of b: a shared FP64 atomic is a loop of compare-and-
+      // swaps that takes the lanes one by one, so from six exits on they are
+      // summed across the warp first (11-step paths, eight exits at a time:
+      // 10.3 -> 8.2 ms; the extended kernels gather four).
+      if (!EXT && __popc(m) > 5) {
+        const double sum = warp_sum((m >> lane) & 1 ? bc : 0.0);
+        if (lane == 0) atomicAdd(&S.st(s).bsum, sum);
+      } else if ((m >> lane) & 1) {
+        atomicAdd(&S.st(s).bsum, bc);
+      }
+      __syncwarp();
       __threadfence_block();
       int fin = 0;
       if (lane == 0) {

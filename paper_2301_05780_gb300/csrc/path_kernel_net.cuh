@@ -528,6 +528,7 @@ __global__ void __launch_bounds__(kNetRows, 5)
       const int s = __shfl_sync(kFull, st, __ffs(gone) - 1);
       const unsigned m = __ballot_sync(kFull, st == s) & gone;
       gone &= ~m;
+      __syncwarp();
       __threadfence_block();
       int fin = 0;
       if (lane == 0) {

@@ -442,8 +442,10 @@ struct LaunchPlan {
 //    within 1 %); where shared memory limits the CTAs (coefficient tiles, wide
 //    stencils) more warps have to share one (tabulated fields, three CTAs per
 //    SM: 31 ms with 192 or 256 threads, 57 with 64, 38 with 384);
-//  - exit batch: 4 lanes, 8 where a path takes fewer steps than two visits of
-//    the step loop (2 % on paths of 11 steps, 2-4 % slower on long ones).
+//  - exit batch: 4 lanes; where a path takes fewer than 16 steps, and resolving
+//    exits takes as long as stepping, 16 (paths of 11 steps: 8.2 ms with 8,
+//    7.65 with 16, 8.5 with 24); 8 in between and for the warpgroup kernel,
+//    whose other lanes wait with the exited ones (8.0 ms with 8, 8.4 with 16).
 pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob, size_t sbytes,
                         double dt, int64_t units, LaunchPlan& L) {
   // cv 3: the in-path network on tcgen05 (the warpgroup kernel)
@@ -505,7 +507,8 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
   CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, L.smem));
   L.grid = c->num_sms * per_sm;
   L.unit_paths = c->auto_unit ? 0 : c->unit_paths;
-  L.exit_batch = !c->auto_batch ? c->exit_batch : mean_steps_estimate(c, dt) < 32.0 ? 8 : 4;
+  const double steps = mean_steps_estimate(c, dt);
+  L.exit_batch = !c->auto_batch ? c->exit_batch : steps < 16.0 && L.cv != 3 ? 16 : steps < 32.0 ? 8 : 4;
   return PDDS_OK;
 }
 
