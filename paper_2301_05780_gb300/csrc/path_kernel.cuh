@@ -558,7 +558,7 @@ __device__ __forceinline__ void cv_table_grad(const ProbDesc& D, float x, float 
 // [CV = 2: xi -= Y s grad u0 . dW (Eq. 37)], with dW = -sqrt(h) g for the
 // packed pair g of box_muller4.  The pairs (Z, S) and (X, Y) are updated with
 // packed FP32 instructions; the values are those of the scalar forms.
-template <int COEF, int CV>
+template <int COEF, int CV, bool EXT>
 __device__ __forceinline__ void em_step(const Stage& H, const float* tile, const KParams& P,
                                         bool direct, float xk, float yk, float h, float hl2,
                                         float sqh, float2 g, float& X, float& Y, float& Sx,
@@ -569,9 +569,15 @@ __device__ __forceinline__ void em_step(const Stage& H, const float* tile, const
   float Yw = 1.0f;
   if constexpr (has_c<COEF>()) {
     Yw = ex2_approx(Sx);
-    const float2 zs = fma2(f2(-f * Yw, c), f2(h, hl2), f2(Z, Sx));  // dZ = -f Y dt, dS = c dt
-    Z = zs.x;
-    Sx = zs.y;
+    if constexpr (EXT && COEF == PDDS_COEF_VARSIGMA) {
+      // c = -1 and a step per knot: h log2(e) and the sum in one rounding
+      Z = fmaf(-f * Yw, h, Z);
+      Sx = fmaf(-1.44269504088896341f, h, Sx);
+    } else {
+      const float2 zs = fma2(f2(-f * Yw, c), f2(h, hl2), f2(Z, Sx));  // dZ = -f Y dt, dS = c dt
+      Z = zs.x;
+      Sx = zs.y;
+    }
   } else if constexpr (has_f<COEF>()) {
     Z = fmaf(-f, h, Z);  // c = 0: Y = 1
   }
@@ -635,11 +641,11 @@ template <int COEF, int CV, bool EXT, bool DIRECT>
 __device__ __forceinline__ void step_pair(const PathConst& c, const KParams& P, float2 gA, float2 gB,
                                           PathState& s) {
   float X1 = s.X, Y1 = s.Y, S1 = s.S, Z1 = s.Z, XI1 = s.XI;
-  em_step<COEF, CV>(*c.H, c.tile, P, DIRECT, c.xk, c.yk, c.h, c.hl2, c.sqh, gA, X1, Y1, S1, Z1, XI1);
+  em_step<COEF, CV, EXT>(*c.H, c.tile, P, DIRECT, c.xk, c.yk, c.h, c.hl2, c.sqh, gA, X1, Y1, S1, Z1, XI1);
   const bool e1 = left_patch<COEF, EXT>(*c.H, c.tile, c.xk, c.yk, X1, Y1, c.bx0, c.bx1, c.by0, c.by1,
                                         c.gmc, DIRECT);
   s.X = X1; s.Y = Y1; s.S = S1; s.Z = Z1; s.XI = XI1;
-  em_step<COEF, CV>(*c.H, c.tile, P, DIRECT, c.xk, c.yk, c.h, c.hl2, c.sqh, gB, s.X, s.Y, s.S, s.Z,
+  em_step<COEF, CV, EXT>(*c.H, c.tile, P, DIRECT, c.xk, c.yk, c.h, c.hl2, c.sqh, gB, s.X, s.Y, s.S, s.Z,
                     s.XI);
   const bool e2 = left_patch<COEF, EXT>(*c.H, c.tile, c.xk, c.yk, s.X, s.Y, c.bx0, c.bx1, c.by0,
                                         c.by1, c.gmc, DIRECT);
@@ -689,7 +695,7 @@ __device__ __forceinline__ void step_calls(const PathConst& c, const KParams& P,
       float2 gA, gB;
       box_muller4(r, gA, gB);
       auto step = [&](float2 g) {
-        em_step<COEF, CV>(*c.H, c.tile, P, DIRECT, c.xk, c.yk, c.h, c.hl2, c.sqh, g, s.X, s.Y, s.S, s.Z,
+        em_step<COEF, CV, EXT>(*c.H, c.tile, P, DIRECT, c.xk, c.yk, c.h, c.hl2, c.sqh, g, s.X, s.Y, s.S, s.Z,
                           s.XI);
         ++s.n;
         s.exited = left_patch<COEF, EXT>(*c.H, c.tile, c.xk, c.yk, s.X, s.Y, c.bx0, c.bx1, c.by0,
