@@ -427,7 +427,8 @@ int64_t default_kmax(const pdds_ctx* c, double dt) {
   return (int64_t)std::ceil(40.0 * T / dt);
 }
 
-// The shape of one path-kernel launch (units: at least so many it will have).
+// The shape of one path-kernel launch (units: at least so many it will have;
+// per_knot: the uniform budget, or 0).
 struct LaunchPlan {
   int cv = 0, block = 0, grid = 0, exit_batch = 0, stages = 2;
   size_t smem = 0;
@@ -447,7 +448,7 @@ struct LaunchPlan {
 //    7.65 with 16, 8.5 with 24); 8 in between and for the warpgroup kernel,
 //    whose other lanes wait with the exited ones (8.0 ms with 8, 8.4 with 16).
 pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob, size_t sbytes,
-                        double dt, int64_t units, LaunchPlan& L) {
+                        double dt, int64_t units, int64_t per_knot, LaunchPlan& L) {
   // cv 3: the in-path network on tcgen05 (the warpgroup kernel)
   L.cv = nprob == 1 ? c->cv_mode : 0;
   if (L.cv == 1 && c->net_engine == PDDS_NET_TCGEN05) L.cv = 3;
@@ -502,6 +503,26 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
       L.stages = r;
       L.smem = smem;
       break;
+    }
+  }
+  // Coefficient tiles that leave room for two stages only: fewer, larger CTAs
+  // of three stages keep as many warps and wait less for a unit's last paths,
+  // once units are long enough to be worth sharing (1,000 paths per knot 31.25 ->
+  // 30.05 ms, 2,000 4.34 -> 4.24; 300: 8.54 -> 8.74, so not below 512).
+  if (coef_id == PDDS_COEF_TABLE && L.stages == 2 && L.cv != 1 && c->auto_block &&
+      c->ctas_per_sm <= 0 && per_knot >= 512) {
+    const int block = 384;
+    const size_t smem = 3 * sbytes + net;
+    int ctas = 0;
+    if (2 * smem <= 227 * 1024) {
+      CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, smem));
+      CK(c, pdds::path_kernel_occupancy(coef_id, rec, L.cv, ext, block, smem, &ctas));
+    }
+    if (ctas == 2 && units >= 3 * 2 * (int64_t)c->num_sms) {
+      L.block = block;
+      L.stages = 3;
+      L.smem = smem;
+      per_sm = ctas;
     }
   }
   CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, L.smem));
@@ -605,7 +626,9 @@ pdds_status assemble_impl(pdds_ctx* c, const int64_t* N, int64_t Nu, double dt, 
   const bool gm = (scheme < 0 ? c->scheme : scheme) == PDDS_SCHEME_GM;
   const bool ext = gm || c->d_hknot != nullptr || c->interp == PDDS_INTERP_RBF;
   LaunchPlan L;
-  if (pdds_status e = plan_launch(c, c->coef_id, rec != nullptr, ext, 1, stage_bytes(c), dt, c->geo.n, L)) return e;
+  if (pdds_status e = plan_launch(c, c->coef_id, rec != nullptr, ext, 1, stage_bytes(c), dt, c->geo.n,
+                                    N ? 0 : Nu, L))
+    return e;
   ProbDesc D = make_prob(c, (int)c->tag);
   D.Gval = G->val;
   D.b = b;
@@ -1443,7 +1466,7 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
       return round_up(x, 128);
     }();
     LaunchPlan L;
-    if (pdds_status e = plan_launch(c0, c0->coef_id, false, false, count == 1 ? 1 : 2, sb, dt, knots, L))
+    if (pdds_status e = plan_launch(c0, c0->coef_id, false, false, count == 1 ? 1 : 2, sb, dt, knots, 0, L))
       return e;
     std::vector<ProbDesc> probs(count);
     for (int i = 0; i < count; ++i) {

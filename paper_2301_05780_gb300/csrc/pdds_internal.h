@@ -65,7 +65,7 @@ struct ProbDesc {
   const int64_t* rbf_off;         // [2][rbf_lmax + 1] table offset per (orientation, length)
   int32_t rbf_lmax;
   int32_t cv_nx;                  // tabulated control variate: nodes per row, or 0
-  const float* cv_tab;            // [cv_ny][cv_nx][2] grad u0 spanning Omega, or nullptr
+  const float* cv_tab;            // grad u0 by cell: [cv_ny-1][cv_nx-1][4 corners][2], or nullptr
   int32_t cv_ny;
   float cv_inv_dx, cv_inv_dy;     // table nodes per unit length
   int32_t pad1_;
@@ -133,7 +133,7 @@ bool path_kernel_has_cv(int coef_id);
 size_t mlp_image_bytes();
 cudaError_t mlp_stage(const float* theta, void* image, cudaStream_t stream);
 // The paths of a work unit for a launch of `paths` paths on `ctas` resident
-// CTAs of `warps` warps, when the caller has set none.  A CTA holds two units
+// CTAs of `warps` warps, when the caller has set none.  A CTA holds two or more units
 // at a time, so its lanes stay full only with units of about its lanes, and
 // its last units bound the launch's tail:
 //  - several waves of lanes: 2.5 units per CTA, within one and eight waves of
