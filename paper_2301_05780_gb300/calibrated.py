@@ -88,7 +88,7 @@ def run(w: W.Workload, eps: float, n0: int, h0: float, n_job: int, n0p: int | No
     the library's default (256, 4096, 4).  The default here was measured on
     the paper's problem, one GB300, over 15 shapes: 152 ms per pipeline
     against 173 ms with the library's default (budgets of ~1,300 paths per
-    knot fill units of 1024 and give each CTA's two-stage ring short units).
+    knot fill units of 1024 and give each CTA's ring short units).
     Returns the nodal solutions of Phases I and III, the calibration (h_i,
     N_i, gap, var, rho^2), per-phase wall times (CUDA-synchronized) and
     path-step counts."""

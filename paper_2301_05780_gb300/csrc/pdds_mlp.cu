@@ -584,12 +584,12 @@ pdds_status train_impl(int engine, const char* name, float* theta, const float* 
       pa.persistent = 1;
       void* args[] = {&pa};
       r = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(threads), args, smem, s);
-      if (r != cudaErrorCooperativeLaunchTooLarge) {
-        if (r == cudaSuccess && loss_history_host)
+      if (r == cudaSuccess) {
+        if (loss_history_host)
           r = cudaMemcpyAsync(loss_history_host, a.loss, steps * sizeof(double),
                               cudaMemcpyDeviceToHost, s);
-        if (r == cudaSuccess) r = cudaStreamSynchronize(s);
-        return r;
+        const cudaError_t done = cudaStreamSynchronize(s);
+        return r != cudaSuccess ? r : done;
       }
       (void)cudaGetLastError();
     }
@@ -638,7 +638,7 @@ pdds_status train_impl(int engine, const char* name, float* theta, const float* 
   };
   cudaError_t e = run();
   // (also after a failure: the buffer goes back only when nothing uses it)
-  if (e != cudaSuccess) (void)cudaStreamSynchronize(s);
+  if (e != cudaSuccess) (void)cudaDeviceSynchronize();
   if (e != cudaSuccess) return mlp_cuda(e, name);
   return PDDS_OK;
 }

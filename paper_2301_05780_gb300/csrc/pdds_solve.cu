@@ -30,6 +30,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <mutex>
 #include <string>
@@ -61,7 +62,7 @@ struct SolveDesc {
   const double* b;
   double* x;
   double* work;       // r, rh, p, v, s, t: 6 n
-  SolveScalars* sc;   // zeroed before the launch
+  SolveScalars* sc;   // up to the partial sums zeroed before the launch
   int64_t n;
   double rtol;
   uint64_t wait_ns;   // bound on a barrier's wait
@@ -348,12 +349,19 @@ cudaError_t bicgstab_batch(SolveJob* jobs, int count, double rtol, int32_t maxit
         ctas += D.ctas;
       }
       for (int i = 0; i < P.count; ++i)
-        if ((e = cudaMemsetAsync(P.inl[i].sc, 0, sizeof(SolveScalars), st)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(P.inl[i].sc, 0, offsetof(SolveScalars, part), st)) != cudaSuccess)
+          return e;
       void* args[] = {&P};
-      e = cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_bicgstab), dim3(ctas), dim3(kThreads),
-                                      args, 0, st);
-      // fewer SMs than the device has (a partition): a smaller team
-      if (e == cudaErrorCooperativeLaunchTooLarge && limit > 1) { (void)cudaGetLastError(); continue; }
+      // one CTA per problem: none waits for another, an ordinary launch will do
+      const void* fn = reinterpret_cast<const void*>(k_bicgstab);
+      e = ctas == P.count ? cudaLaunchKernel(fn, dim3(ctas), dim3(kThreads), args, 0, st)
+                          : cudaLaunchCooperativeKernel(fn, dim3(ctas), dim3(kThreads), args, 0, st);
+      // fewer SMs than the device has (a partition), or no cooperative
+      // launches: smaller teams, in the end of one CTA each
+      if ((e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) && limit > 1) {
+        (void)cudaGetLastError();
+        continue;
+      }
       if (e != cudaSuccess) return e;
       break;
     }

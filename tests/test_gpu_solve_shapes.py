@@ -58,3 +58,63 @@ def test_zero_right_hand_side_and_maxit():
     with pytest.raises(pdds.PddsError) as e:
         pdds.pdds_solve_noalloc(G, dev(b), u, rtol=1e-14, maxit=2)
     assert e.value.status == pdds.PDDS_ENOCONV and "after 2 iterations" in str(e.value)
+
+
+def test_solves_and_fits_from_several_threads():
+    """The solve and the tensor-core fit are cooperative launches whose CTAs wait
+    for one another: several of them at once, on streams of their own next to
+    assemblies, all finish, and every solve gives the serial result bit for bit."""
+    import threading
+
+    from paper_2301_05780_gb300 import workloads as W
+
+    ws = [W.config1(), W.config2().scaled(n_paths=300), W.paper_e1().scaled(n_paths=20)]
+    probs = [pdds.Problem(w) for w in ws]
+    want = []
+    for P in probs:
+        P.assemble()
+        P.solve()
+        want.append(P.u.clone())
+    busy = pdds.Problem(W.config2().scaled(n_paths=2000))
+    xy = torch.rand(11_000, 2, device="cuda") * 2 - 1
+    t = torch.sin(3 * xy[:, 0]) * xy[:, 1]
+    torch.cuda.synchronize()
+    bad = []
+
+    def solve(i):
+        s = torch.cuda.Stream()
+        for _ in range(25):
+            u = torch.full_like(want[i], float("nan"))
+            torch.cuda.current_stream().synchronize()
+            pdds.pdds_solve(probs[i].ctx, probs[i].G, probs[i].b, u, 1e-12, 5000, stream=s)
+            if not torch.equal(u, want[i]):
+                bad.append(("solve", i))
+
+    def fit():
+        s = torch.cuda.Stream()
+        for _ in range(10):
+            th = torch.tensor(W.mlp_init(), dtype=torch.float32, device="cuda")
+            torch.cuda.current_stream().synchronize()
+            loss = pdds.pdds_mlp_train(th, xy, t, steps=20, stream=s, engine="tc")
+            if not (np.isfinite(loss).all() and loss[-1] < loss[0]):
+                bad.append(("fit", loss))
+
+    def assemble():
+        s = torch.cuda.Stream()
+        for _ in range(10):
+            busy.assemble(stream=s)
+            s.synchronize()
+
+    def guard(f, *a):
+        def run():
+            try:
+                f(*a)
+            except Exception as e:   # a wait that ran out comes back as an error
+                bad.append((f.__name__, repr(e)))
+        return run
+
+    ts = [threading.Thread(target=guard(solve, i)) for i in range(3)] + \
+         [threading.Thread(target=guard(f)) for f in (fit, fit, assemble)]
+    [x.start() for x in ts]
+    [x.join() for x in ts]
+    assert not bad, bad[:3]
