@@ -1167,12 +1167,16 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
   S.qempty = &s_qempty;
   const int64_t total_units = P.prob_unit_prefix[P.nprob];
   int units_done = 0;
+  // No more units than CTAs: one each, or the first CTAs would take two or three
+  // and the others none (long paths in a few large units: twice the time).
+  const int load_stages = total_units <= (int64_t)gridDim.x ? 1 : P.stages;
   if (threadIdx.x == 0) {
     s_live = 0;
     s_qempty = 0;
     for (int s = 0; s < P.stages; ++s) {
-      S.st(s).ctrl = 1ull << 32;  // "loading its unit 0"
-      S.st(s).term = 0;
+      const bool used = s < load_stages;
+      S.st(s).ctrl = used ? 1ull << 32 : 0ull;  // "loading its unit 0", or published and terminal
+      S.st(s).term = used ? 0 : 1;
       S.st(s).tma_phase = 0;
       mbar_init(&S.st(s).mbar);
     }
@@ -1180,7 +1184,7 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
   }
   __syncthreads();
   bool ok = true;
-  for (int s = warp; s < P.stages && ok; s += (int)(blockDim.x >> 5))
+  for (int s = warp; s < load_stages && ok; s += (int)(blockDim.x >> 5))
     ok = load_unit<EXT>(S, s, 0, P, total_units, units_done);
   __syncthreads();
 

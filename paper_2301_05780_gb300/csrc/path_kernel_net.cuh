@@ -288,12 +288,16 @@ __global__ void __launch_bounds__(kNetRows, 5)
   S.qempty = &s_qempty;
   const int64_t total_units = P.prob_unit_prefix[P.nprob];
   int units_done = 0;
+  // No more units than CTAs: one each, or the first CTAs would take two or three
+  // and the others none (long paths in a few large units: twice the time).
+  const int load_stages = total_units <= (int64_t)gridDim.x ? 1 : P.stages;
   if (tid == 0) {
     s_live = 0;
     s_qempty = 0;
     for (int s = 0; s < P.stages; ++s) {
-      S.st(s).ctrl = 1ull << 32;  // "loading its unit 0"
-      S.st(s).term = 0;
+      const bool used = s < load_stages;
+      S.st(s).ctrl = used ? 1ull << 32 : 0ull;  // "loading its unit 0", or published and terminal
+      S.st(s).term = used ? 0 : 1;
       S.st(s).tma_phase = 0;
       mbar_init(&S.st(s).mbar);
     }
@@ -308,7 +312,7 @@ __global__ void __launch_bounds__(kNetRows, 5)
   __syncthreads();
   tc::fence_after();
   bool ok = true;
-  for (int s = warp; s < P.stages && ok; s += kNetRows / 32)
+  for (int s = warp; s < load_stages && ok; s += kNetRows / 32)
     ok = load_unit<EXT>(S, s, 0, P, total_units, units_done);
   __syncthreads();
   const unsigned tm = N.tmem, ts = N.tmem_s1;
