@@ -458,7 +458,7 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
                      : L.cv == 3 ? pdds::net_smem_bytes()
                                  : 0;
   L.smem = 2 * sbytes + net;
-  CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, L.smem));
+  CK(c, pdds::allow_path_kernel_smem(coef_id, rec, L.cv, ext, L.smem));
   int per_sm = 0;
   if (L.cv == 3) {
     L.block = 128;  // one warpgroup
@@ -497,7 +497,7 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
     const int64_t ctas_all = (int64_t)c->num_sms * per_sm;
     if (units < r * ctas_all || smem * per_sm > (size_t)(L.cv == 2 ? 160 : 227) * 1024) continue;
     int ctas = 0;
-    CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, smem));
+    CK(c, pdds::allow_path_kernel_smem(coef_id, rec, L.cv, ext, smem));
     CK(c, pdds::path_kernel_occupancy(coef_id, rec, L.cv, ext, L.block, smem, &ctas));
     if (ctas >= per_sm) {
       L.stages = r;
@@ -515,7 +515,7 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
     const size_t smem = 3 * sbytes + net;
     int ctas = 0;
     if (2 * smem <= 227 * 1024) {
-      CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, smem));
+      CK(c, pdds::allow_path_kernel_smem(coef_id, rec, L.cv, ext, smem));
       CK(c, pdds::path_kernel_occupancy(coef_id, rec, L.cv, ext, block, smem, &ctas));
     }
     if (ctas == 2 && units >= 3 * 2 * (int64_t)c->num_sms) {
@@ -525,7 +525,6 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
       per_sm = ctas;
     }
   }
-  CK(c, pdds::set_path_kernel_smem(coef_id, rec, L.cv, ext, L.smem));
   L.grid = c->num_sms * per_sm;
   L.unit_paths = c->auto_unit ? 0 : c->unit_paths;
   const double steps = mean_steps_estimate(c, dt);

@@ -127,7 +127,9 @@ cudaError_t launch_path_kernel(int coef_id, bool records, int cv, bool ext, cons
                                int grid, int block, size_t smem, cudaStream_t stream);
 cudaError_t path_kernel_occupancy(int coef_id, bool records, int cv, bool ext, int block,
                                   size_t smem, int* ctas_per_sm);
-cudaError_t set_path_kernel_smem(int coef_id, bool records, int cv, bool ext, size_t smem);
+// Lets launches of the kernel take up to `smem` bytes of dynamic shared memory
+// (before an occupancy query or a launch with that size; never takes any away).
+cudaError_t allow_path_kernel_smem(int coef_id, bool records, int cv, bool ext, size_t smem);
 bool path_kernel_has_cv(int coef_id);
 // Control-variate network (pdds_mlp.cu): FP32 theta -> staged image.
 size_t mlp_image_bytes();

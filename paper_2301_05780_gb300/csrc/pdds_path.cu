@@ -5,8 +5,10 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
-#include <algorithm>
 #include <stdint.h>
+
+#include <algorithm>
+#include <mutex>
 
 #include "pdds.h"
 #include "pdds_internal.h"
@@ -160,13 +162,23 @@ cudaError_t path_kernel_occupancy(int coef, bool rec, int cv, bool ext, int bloc
   return cudaSuccess;
 }
 
-cudaError_t set_path_kernel_smem(int coef, bool rec, int cv, bool ext, size_t smem) {
+// The attribute belongs to the kernel on the device, not to a context or a
+// thread: another thread may launch the same kernel between this call and the
+// caller's launch.  So it is only ever raised, under a lock, from what the
+// device itself reports (nothing to go stale); launches and occupancy queries
+// take the size they use as an argument.
+cudaError_t allow_path_kernel_smem(int coef, bool rec, int cv, bool ext, size_t smem) {
   void* fn = pick(coef, rec, cv, ext);
   if (!fn) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  // the tcgen05 network kernel (~55 KB per CTA) needs the large shared-memory
-  // carve-out for two CTAs per SM
-  if (e == cudaSuccess && cv == 3)
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lock(mu);
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+  if (e == cudaSuccess && (size_t)fa.maxDynamicSharedSizeBytes < smem)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the tcgen05 network kernel (about 45 KB per CTA with two stages) needs the
+  // large shared-memory carve-out for its five CTAs per SM
+  if (e == cudaSuccess && cv == 3 && fa.preferredShmemCarveout != (int)cudaSharedmemCarveoutMaxShared)
     e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
   return e;
