@@ -668,14 +668,33 @@ __device__ __forceinline__ void step_pair(const PathConst& c, const KParams& P, 
 // 48.5 -> 46.9 ms at 1.4e10 path-steps, variable sigma 466 -> 461 ms at
 // 1.5e11, the paper's GM warm-up, until then one branch per step, 20.1 -> 18.9
 // ms at 4.4e9, its production run 46.9 -> 45.3 ms).
-template <int COEF, int CV, bool EXT, bool DIRECT>
+// MIXED: a path of the mixed run resumes after its Gobet-Menozzi exit at any
+// step.  At an odd one it first takes the second half of its call by itself, so
+// that the lanes of a warp share the loop that follows (with the whole visit
+// step by step, warps paid for both loops: calibration of the paper's problem
+// 35.3 -> 33.6 ms; of 1.6e6 paths of 60 steps 1.60 -> 1.46 ms, and 1.42 without
+// the idle lanes' draws, which is what one loop for every step had taken).
+template <int COEF, int CV, bool EXT, bool DIRECT, bool MIXED>
 __device__ __forceinline__ void step_calls(const PathConst& c, const KParams& P, const PhiloxPath& ph,
                                            int kmax, PathState& s, bool& trunc) {
   constexpr bool kPre = EXT && CV == 0;
   // (the tabulated set's extended kernel spills more with two exact exit tests
   // per call: 2 % slower, so it goes step by step)
   constexpr bool kPair = !(EXT && COEF == PDDS_COEF_TABLE);
-  if (kPair && !(s.n & 1) && s.n + 2 * P.calls_per_check < kmax) {
+  if constexpr (MIXED && kPair) {
+    if (s.n & 1) {
+      const uint4 r = philox4x32_10(make_uint4((uint32_t)(s.n >> 1), c.p, c.kk, c.tagw), P.round_keys);
+      float2 gA, gB;
+      box_muller4(r, gA, gB);
+      em_step<COEF, CV, EXT>(*c.H, c.tile, P, DIRECT, c.xk, c.yk, c.h, c.hl2, c.sqh, gB, s.X, s.Y, s.S,
+                             s.Z, s.XI);
+      ++s.n;
+      s.exited = left_patch<COEF, EXT>(*c.H, c.tile, c.xk, c.yk, s.X, s.Y, c.bx0, c.bx1, c.by0,
+                                       c.by1, c.gmc, DIRECT);
+      if (!s.exited && s.n >= kmax) { s.exited = true; trunc = true; }
+    }
+  }
+  if (kPair && s.n + 2 * P.calls_per_check < kmax) {
 #pragma unroll 1
     for (int call = P.calls_per_check; call > 0 && !s.exited; --call) {
       const uint4 r = kPre ? philox_step((uint32_t)(s.n >> 1), ph, P.round_keys)
@@ -686,7 +705,7 @@ __device__ __forceinline__ void step_calls(const PathConst& c, const KParams& P,
       step_pair<COEF, CV, EXT, DIRECT>(c, P, gA, gB, s);
     }
   } else {
-    // step by step: near the step cap, or resuming a mixed run at an odd step
+    // step by step: near the step cap
 #pragma unroll 1
     for (int call = P.calls_per_check; call > 0 && !s.exited; --call) {
       const uint4 r = kPre && !kPair ? philox_step((uint32_t)(s.n >> 1), ph, P.round_keys)
@@ -702,11 +721,11 @@ __device__ __forceinline__ void step_calls(const PathConst& c, const KParams& P,
                                          c.by1, c.gmc, DIRECT);
         if (!s.exited && s.n >= kmax) { s.exited = true; trunc = true; }
       };
-      // a call serves steps 2q and 2q + 1; a path that resumes at an odd step
-      // takes the second half of its call
+      // a call serves steps 2q and 2q + 1 (the tabulated set's mixed run comes
+      // here at an odd step too)
       if constexpr (kPair) {
 #pragma unroll 1
-        for (int half = s.n & 1; half < 2 && !s.exited; ++half) step(half ? gB : gA);
+        for (int half = 0; half < 2 && !s.exited; ++half) step(half ? gB : gA);
       } else {
         if (!(s.n & 1)) step(gA);
         if (!s.exited) step(gB);
@@ -1361,15 +1380,18 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
         const int m = __popc(todo), log2g = m > 1 ? __clz(m - 1) - 27 : 5;  // 32 / m paths, rounded down
         const int rounds = max(1, P.calls_per_check >> log2g);
         // (not for the tabulated set: its steps wait for shared-memory lookups,
-        // not for Philox, and ran 6 % slower this way)
-        if (COEF != PDDS_COEF_TABLE && log2g > 0 && todo != 0 &&
+        // not for Philox, and ran 6 % slower this way; nor for the mixed run's
+        // kernels, whose resumed paths are at odd steps half of the time and
+        // whose loops spill more beside it: the paper's calibration 33.6 -> 32.5
+        // ms without)
+        if (COEF != PDDS_COEF_TABLE && !kMixed && log2g > 0 && todo != 0 &&
             __all_sync(kFull, !((todo >> lane) & 1) ||
                                   (!(n & 1) && n + ((2 * rounds) << log2g) < kmax))) {
           if (kAngles && P.trig_direct) coop_calls<COEF, CV, EXT, kAngles>(c, P, todo, log2g, rounds, s);
           else coop_calls<COEF, CV, EXT, false>(c, P, todo, log2g, rounds, s);
         } else if (alive && !exited) {
-          if (kAngles && P.trig_direct) step_calls<COEF, CV, EXT, kAngles>(c, P, ph, kmax, s, trunc);
-          else step_calls<COEF, CV, EXT, false>(c, P, ph, kmax, s, trunc);
+          if (kAngles && P.trig_direct) step_calls<COEF, CV, EXT, kAngles, kMixed>(c, P, ph, kmax, s, trunc);
+          else step_calls<COEF, CV, EXT, false, kMixed>(c, P, ph, kmax, s, trunc);
         }
         X = s.X; Y = s.Y; Sx = s.S; Z = s.Z; XI = s.XI; n = s.n; exited = s.exited;
       }
