@@ -534,6 +534,9 @@ __device__ __forceinline__ const ProbDesc& prob_desc(const KParams& P, int i) {
 // loads from two rows (7 % faster per step on the paper's problem).  Both
 // components are interpolated at once in packed FP32 (six instructions instead
 // of twelve), and the weights are clamped by the subtraction's saturation.
+// PACKED = false: one component after the other, the same values (the E1 set's
+// naive-exit kernel, whose registers the pairs press: 4 % faster).
+template <bool PACKED>
 __device__ __forceinline__ void cv_table_grad(const ProbDesc& D, float x, float y, float& gx,
                                               float& gy) {
   const float fx = (x - D.x0) * D.cv_inv_dx, fy = (y - D.y0) * D.cv_inv_dy;
@@ -544,6 +547,13 @@ __device__ __forceinline__ void cv_table_grad(const ProbDesc& D, float x, float 
   // (at most 2^28 nodes: the cell index fits 32 bits)
   const float4* cell = reinterpret_cast<const float4*>(D.cv_tab) + 2 * (int64_t)(j * (D.cv_nx - 1) + i);
   const float4 G = __ldg(cell), H = __ldg(cell + 1);
+  if constexpr (!PACKED) {
+    const float x0 = fmaf(tx, G.z - G.x, G.x), x1 = fmaf(tx, H.z - H.x, H.x);
+    const float y0 = fmaf(tx, G.w - G.y, G.y), y1 = fmaf(tx, H.w - H.y, H.y);
+    gx = fmaf(ty, x1 - x0, x0);
+    gy = fmaf(ty, y1 - y0, y0);
+    return;
+  }
   const float2 n00 = f2(G.x, G.y), n01 = f2(G.z, G.w), n10 = f2(H.x, H.y), n11 = f2(H.z, H.w);
   const float2 m1 = f2(-1.0f, -1.0f);
   const float2 b = fma2(f2(tx, tx), fma2(n00, m1, n01), n00);
@@ -586,7 +596,7 @@ __device__ __forceinline__ void em_step(const Stage& H, const float* tile, const
     // grad u0 from the table; a control variate never runs batched, so the
     // table is problem 0's, read from the launch constants
     float gx, gy;
-    cv_table_grad(P.prob0, a.x, a.y, gx, gy);
+    cv_table_grad<EXT || COEF != PDDS_COEF_POISSON_E1>(P.prob0, a.x, a.y, gx, gy);
     XI = fmaf(Yw * ssh, fmaf(gx, g.x, gy * g.y), XI);
   }
   float2 p = f2(X, Y);
@@ -668,12 +678,48 @@ __device__ __forceinline__ void step_pair(const PathConst& c, const KParams& P, 
 // 48.5 -> 46.9 ms at 1.4e10 path-steps, variable sigma 466 -> 461 ms at
 // 1.5e11, the paper's GM warm-up, until then one branch per step, 20.1 -> 18.9
 // ms at 4.4e9, its production run 46.9 -> 45.3 ms).
+// With the tabulated control variate on the naive exit, the sets whose own step
+// leaves no registers for that form (the tabulated one and E1: 84 and 48 bytes
+// of spills against 0 and 12) keep the selects and compares (step_selects):
+// E1 at 60 steps a path 1.04 -> 0.96 ms per 1.6e6 paths, tabulated at 400 steps
+// 1.50 -> 1.44 ms per 5,800 paths, 15.6 -> 15.1 ms per 2.5e6.
 // MIXED: a path of the mixed run resumes after its Gobet-Menozzi exit at any
 // step.  At an odd one it first takes the second half of its call by itself, so
 // that the lanes of a warp share the loop that follows (with the whole visit
 // step by step, warps paid for both loops: calibration of the paper's problem
 // 35.3 -> 33.6 ms; of 1.6e6 paths of 60 steps 1.60 -> 1.46 ms, and 1.42 without
 // the idle lanes' draws, which is what one loop for every step had taken).
+template <int COEF, int CV, bool EXT>
+__host__ __device__ constexpr bool uses_selects() {
+  return !EXT && CV == 2 && (COEF == PDDS_COEF_TABLE || COEF == PDDS_COEF_POISSON_E1);
+}
+template <int COEF, int CV, bool DIRECT>
+__device__ __forceinline__ void step_selects(const PathConst& c, const KParams& P, int kmax,
+                                             PathState& s, bool& trunc) {
+#pragma unroll 1
+  for (int call = P.calls_per_check; call > 0 && !s.exited; --call) {
+    const uint4 r = philox4x32_10(make_uint4((uint32_t)(s.n >> 1), c.p, c.kk, c.tagw), P.round_keys);
+    float2 gA, gB;
+    box_muller4(r, gA, gB);
+    PathState s1 = s;
+    em_step<COEF, CV, false>(*c.H, c.tile, P, DIRECT, c.xk, c.yk, c.h, c.hl2, c.sqh, gA, s1.X, s1.Y,
+                             s1.S, s1.Z, s1.XI);
+    s1.exited = outside_box(s1.X, s1.Y, c.bx0, c.bx1, c.by0, c.by1);
+    PathState s2 = s1;
+    em_step<COEF, CV, false>(*c.H, c.tile, P, DIRECT, c.xk, c.yk, c.h, c.hl2, c.sqh, gB, s2.X, s2.Y,
+                             s2.S, s2.Z, s2.XI);
+    s2.exited = outside_box(s2.X, s2.Y, c.bx0, c.bx1, c.by0, c.by1);
+    const bool first = s1.exited || s.n + 1 >= kmax;
+    s.X = first ? s1.X : s2.X;
+    s.Y = first ? s1.Y : s2.Y;
+    s.S = first ? s1.S : s2.S;
+    s.Z = first ? s1.Z : s2.Z;
+    s.XI = first ? s1.XI : s2.XI;
+    s.n += first ? 1 : 2;
+    s.exited = first ? s1.exited : s2.exited;
+    if (!s.exited && s.n >= kmax) { s.exited = true; trunc = true; }
+  }
+}
 template <int COEF, int CV, bool EXT, bool DIRECT, bool MIXED>
 __device__ __forceinline__ void step_calls(const PathConst& c, const KParams& P, const PhiloxPath& ph,
                                            int kmax, PathState& s, bool& trunc) {
@@ -681,6 +727,10 @@ __device__ __forceinline__ void step_calls(const PathConst& c, const KParams& P,
   // (the tabulated set's extended kernel spills more with two exact exit tests
   // per call: 2 % slower, so it goes step by step)
   constexpr bool kPair = !(EXT && COEF == PDDS_COEF_TABLE);
+  if constexpr (uses_selects<COEF, CV, EXT>()) {
+    step_selects<COEF, CV, DIRECT>(c, P, kmax, s, trunc);
+    return;
+  }
   if constexpr (MIXED && kPair) {
     if (s.n & 1) {
       const uint4 r = philox4x32_10(make_uint4((uint32_t)(s.n >> 1), c.p, c.kk, c.tagw), P.round_keys);
@@ -1379,12 +1429,7 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
         constexpr bool kAngles = uses_angles<COEF>();
         const int m = __popc(todo), log2g = m > 1 ? __clz(m - 1) - 27 : 5;  // 32 / m paths, rounded down
         const int rounds = max(1, P.calls_per_check >> log2g);
-        // (not for the tabulated set: its steps wait for shared-memory lookups,
-        // not for Philox, and ran 6 % slower this way; nor for the mixed run's
-        // kernels, whose resumed paths are at odd steps half of the time and
-        // whose loops spill more beside it: the paper's calibration 33.6 -> 32.5
-        // ms without)
-        if (COEF != PDDS_COEF_TABLE && !kMixed && log2g > 0 && todo != 0 &&
+        if (path_kernel_draws_ahead(COEF, CV, RECORD, EXT) && log2g > 0 && todo != 0 &&
             __all_sync(kFull, !((todo >> lane) & 1) ||
                                   (!(n & 1) && n + ((2 * rounds) << log2g) < kmax))) {
           if (kAngles && P.trig_direct) coop_calls<COEF, CV, EXT, kAngles>(c, P, todo, log2g, rounds, s);

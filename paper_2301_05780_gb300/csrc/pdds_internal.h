@@ -8,6 +8,8 @@
 #include <string>
 #include <vector>
 
+#include "pdds.h"
+
 namespace pdds {
 
 constexpr int kSides = 4;  // patch sides in the order E, N, W, S (Eq. 14)
@@ -134,6 +136,19 @@ bool path_kernel_has_cv(int coef_id);
 // Control-variate network (pdds_mlp.cu): FP32 theta -> staged image.
 size_t mlp_image_bytes();
 cudaError_t mlp_stage(const float* theta, void* image, cudaStream_t stream);
+// Kernels in which the idle lanes of a warp draw normals ahead for its last
+// paths (coop_calls).  Not: the tabulated set, whose steps wait for shared-memory
+// lookups and not for Philox (6 % slower); the mixed run's kernels, whose
+// resumed paths are at odd steps half of the time and whose loops spill more
+// beside it (the paper's calibration 32.5 ms without, 33.6 with); the E1 set but
+// for its extended kernel with the tabulated control variate (its step is long
+// and the shuffles and spills come on top: 3,200 paths of 400 steps 0.49 ms
+// without, 0.57 with; GM exits 0.49 / 0.55; with the table 0.73 / 0.70); the
+// kernels with the in-path network, which step together.
+__host__ __device__ constexpr bool path_kernel_draws_ahead(int coef, int cv, bool records, bool ext) {
+  if (cv == 1 || cv == 3 || coef == PDDS_COEF_TABLE || (ext && records)) return false;
+  return coef != PDDS_COEF_POISSON_E1 || (cv == 2 && ext);
+}
 // The paths of a work unit for a launch of `paths` paths on `ctas` resident
 // CTAs of `warps` warps, when the caller has set none.  A CTA holds two or more units
 // at a time, so its lanes stay full only with units of about its lanes, and
