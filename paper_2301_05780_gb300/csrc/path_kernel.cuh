@@ -1276,7 +1276,7 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
   float xk = 0.f, yk = 0.f, bx0 = 0.f, bx1 = 0.f, by0 = 0.f, by1 = 0.f;
   float X = 0.f, Y = 0.f, Sx = 0.f, Z = 0.f, XI = 0.f;
   unsigned long long my_steps = 0, my_paths = 0, my_trunc = 0, my_clamp = 0;
-  int from = warp % P.stages;  // warp-uniform: the stage the warp takes paths from
+  int from = 0;  // warp-uniform: the stage the warp takes paths from
   // EXT: step, its square root and the step cap of the knot the lane's path
   // belongs to, and the Gobet-Menozzi shift per unit of |s| (0: naive exit);
   // the other variants use the launch constants
@@ -1291,8 +1291,10 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
     for (int guard = 0; idle && guard < 64; ++guard) {
       // Lane s looks at stage s: published, with paths left?  (A hint: the
       // claim below decides.)  Plain kernels: the warp takes the first such
-      // stage from its own starting point on, so that the warps spread over
-      // the ring and its atomics.  Tabulated and extended kernels, whose units
+      // stage from the one it took last on.  (All warps begin with stage 0: if
+      // they begin with different ones, a CTA's units end together and its next
+      // ones are fetched late, all at once; three problems in 4,140 units 58.9
+      // ms, so 63.6.)  Tabulated and extended kernels, whose units
       // are short against their lanes: the stage with the fewest paths left, so
       // that the units end one after the other and not all at once (tabulated
       // 31.8 -> 31.3 ms, paper's production run 42.6 -> 41.8; the plain kernels

@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(kNetRows, 5)
   float xk = 0.f, yk = 0.f, bx0 = 0.f, bx1 = 0.f, by0 = 0.f, by1 = 0.f;
   float X = 0.f, Y = 0.f, Sx = 0.f, Z = 0.f, XI = 0.f;
   unsigned long long my_steps = 0, my_paths = 0, my_trunc = 0, my_clamp = 0;
-  int from = warp % P.stages;
+  int from = 0;
   // EXT: the knot's step, its square root, step cap and Gobet-Menozzi shift
   // per unit of |s|; the mixed GM/EM run of the calibration (records kernels
   // with the extended exit) as in path_kernel
