@@ -976,7 +976,9 @@ __device__ __forceinline__ ExitResult resolve_exit(const Smem& S, const KParams&
 // paper's problem at 200 paths per knot: K = 1 / 2 / 3 / 5 8.9 / 7.3 / 6.9 / 6.6 ms;
 // three, since five cost the same kernel's step loop registers (variable sigma
 // 4 % slower).  The records kernels, whose loop has none to spare (calibration
-// 2.4 % slower with three), keep one.
+// 2.4 % slower with three), keep one, and stencils of up to 32 knots, where the
+// second and third chain would have no knot, take one everywhere (17-knot
+// stencils, 4.3e6 paths of 40 steps: 3.18 ms with three, 3.04 with one).
 template <int COEF, int K>
 __device__ __forceinline__ double rbf_deposit(const Stage& H, unsigned long long* acc, const ProbDesc& D,
                                               int side, float sl, float Y, bool deposit,
@@ -995,24 +997,28 @@ __device__ __forceinline__ double rbf_deposit(const Stage& H, unsigned long long
     return 0.0;
   }
   const int P1 = D.rbf_deg + 1;
-  for (int j0 = lane; j0 < L; j0 += 32 * K) {
-    float w[K];
-    rbf_cardinals<K>(cf, L, P1, j0, tau, w);
+  auto add = [&](int j, float H_j) {
+    const float wj = Y * H_j;
+    const int tl = a + j;
+    if (tl == 0 || tl == lmax) {
+      const int li = vertical ? kd.line[side] : tl;
+      const int lj = vertical ? tl : kd.line[side];
+      dsum += (double)wj * (double)g_value<COEF>(H, fmaf((float)li, H.dx, H.x0),
+                                                 fmaf((float)lj, H.dy, H.y0));
+    } else if (deposit) {
+      // signed weights in 2^-30 units (two's complement in the slot)
+      atomicAdd(acc + kd.off[side] + j, (unsigned long long)__float2ll_rn(wj * kFixedOne));
+    }
+  };
+  if (K == 1 || L <= 32) {  // a knot per lane at most: nothing to take side by side
+    for (int j = lane; j < L; j += 32) add(j, rbf_cardinal(cf, L, P1, j, tau));
+  } else {
+    for (int j0 = lane; j0 < L; j0 += 32 * K) {
+      float w[K];
+      rbf_cardinals<K>(cf, L, P1, j0, tau, w);
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const int j = j0 + 32 * k;
-      if (j >= L) break;
-      const float wj = Y * w[k];
-      const int tl = a + j;
-      if (tl == 0 || tl == lmax) {
-        const int li = vertical ? kd.line[side] : tl;
-        const int lj = vertical ? tl : kd.line[side];
-        dsum += (double)wj * (double)g_value<COEF>(H, fmaf((float)li, H.dx, H.x0),
-                                                   fmaf((float)lj, H.dy, H.y0));
-      } else if (deposit) {
-        // signed weights in 2^-30 units (two's complement in the slot)
-        atomicAdd(acc + kd.off[side] + j, (unsigned long long)__float2ll_rn(wj * kFixedOne));
-      }
+      for (int k = 0; k < K; ++k)
+        if (j0 + 32 * k < L) add(j0 + 32 * k, w[k]);
     }
   }
   return warp_sum(dsum);
