@@ -433,7 +433,14 @@ struct LaunchPlan {
   int cv = 0, block = 0, grid = 0, exit_batch = 0, stages = 2;
   size_t smem = 0;
   int64_t unit_paths = 0;  // 0: auto_unit_paths
-  pdds::UnitRule rule() const { return {grid, block / 32, cv == 3 ? 1 : 0}; }
+  int64_t knots = 1;
+  bool tiles = false;        // a coefficient tile per unit
+  bool draws_ahead = false;  // path_kernel_draws_ahead
+  pdds::UnitRule rule() const {
+    const int64_t warps = block / 32;
+    return {grid, warps, tiles ? grid : grid * std::min<int64_t>(warps, stages), draws_ahead ? 1 : 32,
+            cv == 3 ? 1 : 0, knots};
+  }
 };
 
 // Fields that pdds_set_launch or pdds_autotune have set are kept; the others:
@@ -458,6 +465,9 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
                      : L.cv == 3 ? pdds::net_smem_bytes()
                                  : 0;
   L.smem = 2 * sbytes + net;
+  L.knots = units;
+  L.tiles = coef_id == PDDS_COEF_TABLE;
+  L.draws_ahead = pdds::path_kernel_draws_ahead(coef_id, L.cv, rec, ext);
   CK(c, pdds::allow_path_kernel_smem(coef_id, rec, L.cv, ext, L.smem));
   int per_sm = 0;
   if (L.cv == 3) {

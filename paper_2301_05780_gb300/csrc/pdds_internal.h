@@ -158,17 +158,38 @@ __host__ __device__ constexpr bool path_kernel_draws_ahead(int coef, int cv, boo
 //    2.9e5 paths 2.2 -> 0.6 ms; 1.3e6 1.6 -> 0.75; 1.2e6 variable-sigma paths
 //    7.6 -> 5.3; from 5e6 paths on the upper end is within 1 % of the best);
 //  - fewer paths than lanes: one unit per warp, so that every warp has as few
-//    paths as possible (its idle lanes then draw ahead for them); not for the
-//    warpgroup kernel (whole_ctas), which steps 128 paths at a time.
+//    paths as possible (its idle lanes then draw ahead for them); in the kernels
+//    where they do not, of a warp's lanes at least, since a warp with fewer takes
+//    as long (E1, 30 paths at 1,617 knots, 400 steps: 0.87 ms; 8 a unit 0.98);
+//  - tabulated coefficients (a tile to stage per unit, held until its last path
+//    has left): so few paths in one unit per CTA, of a warp's lanes at least
+//    (30 paths at 833 knots, 400 steps: 1.73 ms; a unit per warp 2.51; 200 paths
+//    at 29 knots 1.44, as with a unit per warp; a unit per knot 1.65);
+//  - the warpgroup kernel steps 128 rows at a time however few of them are
+//    paths, so a unit's last paths cost most: about 1.5 units per CTA of 128 to
+//    512 paths, where a knot's mean budget in equal parts comes near to that, and
+//    knots not worth two units whole (paths of 60 steps, manufactured set, 833
+//    knots at 300 / 1,000 / 2,000 paths: 3.3 / 5.5 / 7.6 ms; units of 4096 3.3 /
+//    6.4 / 11.0; 2.5 units per CTA of up to 1,024 paths, the rest of each knot in
+//    a last one, 3.9 / 5.6 / 8.7).
 struct UnitRule {
   int64_t ctas, warps;
-  int32_t whole_ctas;
+  int64_t spread;  // units of a launch of fewer paths than lanes, at most
+  int64_t least;   // paths of a unit, at least
+  int32_t equal;   // the warpgroup kernel's rule
+  int64_t knots;   // for it: the knots
 };
 __host__ __device__ inline int64_t auto_unit_paths(int64_t paths, const UnitRule& r) {
   const int64_t lo = 32 * r.warps, hi = 256 * r.warps;
-  if (!r.whole_ctas && paths <= r.ctas * lo) {
-    const int64_t u = (paths + r.ctas * r.warps - 1) / (r.ctas * r.warps);
-    return u < 1 ? 1 : u;
+  if (r.equal) {
+    int64_t u = paths * 2 / (3 * r.ctas);
+    u = u < 128 ? 128 : u > 512 ? 512 : u;
+    const int64_t mean = (paths + r.knots - 1) / r.knots, parts = (mean + u / 2) / u;
+    return parts < 2 ? 4096 : (mean + parts - 1) / parts;
+  }
+  if (r.least < lo && paths <= r.ctas * lo) {
+    const int64_t u = (paths + r.spread - 1) / r.spread;
+    return u < r.least ? r.least : u;
   }
   const int64_t u = paths * 2 / (5 * r.ctas);
   return u < lo ? lo : u > hi ? hi : u;
