@@ -450,10 +450,18 @@ struct LaunchPlan {
 //    within 1 %); where shared memory limits the CTAs (coefficient tiles, wide
 //    stencils) more warps have to share one (tabulated fields, three CTAs per
 //    SM: 31 ms with 192 or 256 threads, 57 with 64, 38 with 384);
+//    where they are read through L1 beside the stages (tabulated control variate),
+//    where short stencils leave the warps most to share (RBF) and in the mixed run,
+//    256 for budgets from 512 paths on (E1, 145-knot stencils, 1,600 paths of 40
+//    steps at 26,236 knots 12.0 -> 10.2 ms; at 100 paths 0.81 -> 0.64 with 64);
+//    with the network on mma.sync 128 (11-step paths, manufactured set, 1,000 and
+//    2,000 paths at 833 knots 2.4 and 4.1 ms; 2.6 and 4.3 with 64, 2.5 and 4.2 with 256);
 //  - exit batch: 4 lanes; where a path takes fewer than 16 steps, and resolving
 //    exits takes as long as stepping, 16 (paths of 11 steps: 8.2 ms with 8,
 //    7.65 with 16, 8.5 with 24); 8 in between and for the warpgroup kernel,
-//    whose other lanes wait with the exited ones (8.0 ms with 8, 8.4 with 16).
+//    whose other lanes wait with the exited ones (8.0 ms with 8, 8.4 with 16);
+//    4 with the network on mma.sync, whose every step costs the same for
+//    however many lanes (11-step paths, 2,000 at 833 knots 4.5 ms; 5.1 with 16).
 pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob, size_t sbytes,
                         double dt, int64_t units, int64_t per_knot, LaunchPlan& L) {
   // cv 3: the in-path network on tcgen05 (the warpgroup kernel)
@@ -470,8 +478,8 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
   L.draws_ahead = pdds::path_kernel_draws_ahead(coef_id, L.cv, rec, ext);
   CK(c, pdds::allow_path_kernel_smem(coef_id, rec, L.cv, ext, L.smem));
   int per_sm = 0;
-  if (L.cv == 3) {
-    L.block = 128;  // one warpgroup
+  if (L.cv == 3 || (L.cv == 1 && c->auto_block && c->ctas_per_sm <= 0)) {
+    L.block = 128;  // one warpgroup; the mma.sync network: see above
   } else if (!c->auto_block || c->ctas_per_sm > 0) {
     L.block = L.cv == 1 ? std::min(c->block, 256) : c->block;
   } else {
@@ -483,8 +491,12 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
       warps[i] = ctas * blocks[i] / 32;
       most = std::max(most, warps[i]);
     }
-    for (int i = 3; i >= 0; --i)
+    const bool wide = (per_knot == 0 || per_knot >= 512) &&
+                      (c->interp == PDDS_INTERP_RBF ||
+                       ((L.cv == 2 || (rec && ext)) && mean_steps_estimate(c, dt) >= 32.0));
+    for (int i = 3; i >= (wide ? 3 : 0); --i)
       if (warps[i] >= std::min(most, 24)) L.block = blocks[i];
+    if (L.block == 0) L.block = blocks[std::max_element(warps, warps + 4) - warps];
   }
   per_sm = c->ctas_per_sm;
   if (per_sm <= 0) {
@@ -538,7 +550,10 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
   L.grid = c->num_sms * per_sm;
   L.unit_paths = c->auto_unit ? 0 : c->unit_paths;
   const double steps = mean_steps_estimate(c, dt);
-  L.exit_batch = !c->auto_batch ? c->exit_batch : steps < 16.0 && L.cv != 3 ? 16 : steps < 32.0 ? 8 : 4;
+  L.exit_batch = !c->auto_batch || L.cv == 1      ? c->exit_batch
+                 : steps < 16.0 && L.cv != 3 ? 16
+                 : steps < 32.0              ? 8
+                                             : 4;
   return PDDS_OK;
 }
 
