@@ -5,7 +5,11 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "pdds.h"
+
 namespace pdds {
+
+constexpr uint64_t kTrainWaitNs = 2000000000ull;  // bound on a wait of the tensor-core kernel
 
 // theta = W1[64][2], b1[64], W2[64][64] (row = output unit), b2[64], w3[64], b3
 constexpr int kOffW1 = 0, kOffB1 = 128, kOffW2 = 192, kOffB2 = 4288, kOffW3 = 4352, kOffB3 = 4416;
@@ -33,6 +37,7 @@ struct TrainArgs {
   float lr, beta1, beta2, eps;
   int grad_stride;  // floats between the rotating gradient buffers
   int persistent;   // 1: all steps in one cooperative launch
+  uint64_t mma_ns;  // tensor-core kernel: bound on the wait for a product (0: always run out)
 };
 
 // The tensor-core training kernel (pdds_mlp_train_tc.cu): its function, grid,
@@ -42,3 +47,11 @@ cudaError_t train_tc_launch_config(bool adam, int64_t npts, const void** fn, uns
                                    unsigned* threads, size_t* smem);
 
 }  // namespace pdds
+
+// pdds_mlp_train_tc with a bound of the caller's on the kernel's waits for its
+// products.  Not part of pdds.h: it lets a test make them run out.
+extern "C" pdds_status pdds_internal_mlp_train_tc(float* theta, const float* xy,
+                                                  const float* target, int64_t npts,
+                                                  int32_t steps, double lr,
+                                                  double* loss_history_host, void* cuda_stream,
+                                                  uint64_t mma_ns);

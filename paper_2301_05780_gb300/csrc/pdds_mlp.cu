@@ -514,6 +514,7 @@ pdds_status loss_grad_impl(int engine, const char* name, const float* theta, con
   a.inv_n = 1.0 / (double)npts;
   a.grad = grad;
   a.loss = loss;
+  a.mma_ns = kTrainWaitNs;
   MCK(launch_train(fn, grid, threads, smem, a, s));
   return PDDS_OK;
 }
@@ -534,7 +535,8 @@ extern "C" pdds_status pdds_mlp_loss_grad_tc(const float* theta, const float* xy
 namespace {
 pdds_status train_impl(int engine, const char* name, float* theta, const float* xy,
                        const float* target, int64_t npts, int32_t steps, double lr,
-                       double* loss_history_host, void* cuda_stream) {
+                       double* loss_history_host, void* cuda_stream,
+                       uint64_t mma_ns = kTrainWaitNs) {
   if (!theta || !xy || !target || npts < 1 || steps < 1 || !(lr > 0))
     return mlp_fail(PDDS_EINVAL,
                     std::string(name) + ": NULL pointer, npts < 1, steps < 1 or lr <= 0");
@@ -570,6 +572,7 @@ pdds_status train_impl(int engine, const char* name, float* theta, const float* 
   a.st = reinterpret_cast<TrainState*>(buf + sbytes);
   a.loss = reinterpret_cast<double*>(buf + sbytes + sizeof(TrainState));
   a.steps = steps;
+  a.mma_ns = mma_ns;
   a.lr = (float)lr;
   a.beta1 = 0.9f;
   a.beta2 = 0.999f;
@@ -656,6 +659,15 @@ extern "C" pdds_status pdds_mlp_train_tc(float* theta, const float* xy, const fl
                                          double* loss_history_host, void* cuda_stream) {
   return train_impl(1, "mlp_train_tc", theta, xy, target, npts, steps, lr, loss_history_host,
                     cuda_stream);
+}
+
+extern "C" pdds_status pdds_internal_mlp_train_tc(float* theta, const float* xy,
+                                                  const float* target, int64_t npts,
+                                                  int32_t steps, double lr,
+                                                  double* loss_history_host, void* cuda_stream,
+                                                  uint64_t mma_ns) {
+  return train_impl(1, "mlp_train_tc", theta, xy, target, npts, steps, lr, loss_history_host,
+                    cuda_stream, mma_ns);
 }
 
 extern "C" pdds_status pdds_mlp_eval(const float* theta, const float* xy, int64_t npts, float* v,

@@ -54,7 +54,7 @@ constexpr int kVR = 16;          // rows of the dv tile: dv, zeros
 // TMEM columns: the forward / backward product, SiLU'(a1), the gradient
 // accumulators [g2 | g1]^T [h1 | x | y | 1] and h2^T dv
 constexpr unsigned kColD = 0, kColS1 = 64, kColG = 128, kColW3 = 208, kTmemCols = 256;
-constexpr uint64_t kWaitNs = 2000000000ull;
+constexpr uint64_t kDrainNs = 1000000000ull;
 
 struct alignas(1024) TrainTcSmem {
   uint16_t W2o[kHU * kHU];  // forward B: W2 as N = out x K = in
@@ -170,13 +170,27 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
   const unsigned sP = tc::smem_addr(S.P), sGA = tc::smem_addr(S.GA), sGB = tc::smem_addr(S.GB);
   const unsigned sDV = tc::smem_addr(S.DV);
   unsigned phase = 0;
-  bool ok = true;
+  // ok: no wait of this step has run out.  A product whose wait ran out still
+  // gets kDrainNs to finish, since it reads the operand tiles and writes the
+  // accumulators that the CTA goes on to use and to free; `synced` turns false
+  // for good when it has not, because the barrier's phases then no longer count
+  // the products.
+  bool ok = true, synced = true;
+  auto product_done = [&] {
+    if (A.mma_ns == 0 || !tc::mbar_wait(&S.mbar, phase, A.mma_ns)) {
+      ok = false;
+      synced = tc::mbar_wait(&S.mbar, phase, kDrainNs) && synced;
+    }
+    phase ^= 1u;
+    tc::fence_after();
+  };
   // the points of the CTA's first tile stay in registers over the steps
   const int64_t p0 = (int64_t)blockIdx.x * kTT + pl;
   const float x0 = p0 < A.npts ? A.xy[2 * p0] : 0.f, y0 = p0 < A.npts ? A.xy[2 * p0 + 1] : 0.f;
   const float tg0 = p0 < A.npts ? A.tgt[p0] : 0.f;
   for (;; ++t) {
   const bool grad_pass = !ADAM || t < A.steps;
+  ok = synced;
   if (!ADAM || t == 0) {
     // theta as given; launch 0 of a training run also keeps a copy
     float w_[kPer];
@@ -294,9 +308,7 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
                  false);
       tc::commit(&S.mbar);
     }
-    ok = tc::mbar_wait(&S.mbar, phase, kWaitNs) && ok;
-    phase ^= 1u;
-    tc::fence_after();
+    product_done();
     // ---- output: h2^T (column pl) and the group's part of v; then v, the
     // residual, dv, and g2 into P and g2^T
     float2 us[16];  // u of each unit pair: SiLU'(a2) = (1 + u) / 2
@@ -354,9 +366,7 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
                  false);
       tc::commit(&S.mbar);
     }
-    ok = tc::mbar_wait(&S.mbar, phase, kWaitNs) && ok;
-    phase ^= 1u;
-    tc::fence_after();
+    product_done();
     // ---- g1 = dh1 * SiLU'(a1) into g1^T (column pl)
 #pragma unroll
     for (int qq = 0; qq < 2; ++qq) {
@@ -380,9 +390,7 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
       tc::commit(&S.mbar);
     }
     // the next tile rewrites the operand tiles: wait here
-    ok = tc::mbar_wait(&S.mbar, phase, kWaitNs) && ok;
-    phase ^= 1u;
-    tc::fence_after();
+    product_done();
     ++done;
   }
   if (done > 0) {
@@ -440,7 +448,8 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
       atomicAdd(A.loss + t, l * A.inv_n);
     }
   }
-  if (!ok && tid == 0) atomicAdd(A.loss + t, __longlong_as_double(0x7ff8000000000000ll));
+  // (the last pass only updates: it has no loss)
+  if (!ok && grad_pass && tid == 0) atomicAdd(A.loss + t, __longlong_as_double(0x7ff8000000000000ll));
   if constexpr (!ADAM) {
     break;
   } else if (!A.persistent) {
@@ -471,7 +480,7 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
         if ((spin & 255) == 0) {
           const uint64_t now = tc::now_ns();
           if (began == 0) began = now;
-          if (now - began > kWaitNs) { met = false; break; }
+          if (now - began > kTrainWaitNs) { met = false; break; }
         }
       }
       __threadfence();
