@@ -19,6 +19,9 @@ struct TrainState {
   unsigned count;  // CTAs done with the current launch (persistent: arrivals at the barrier)
   int t;           // index of the next launch
   double p1, p2;   // beta1^t, beta2^t for launch t >= 1
+  // one cooperative launch: 1 once theta holds the last update; 1 once a
+  // barrier's wait has run out (the other CTAs then leave too)
+  int finished, aborted;
 };
 
 struct TrainArgs {
@@ -37,7 +40,9 @@ struct TrainArgs {
   float lr, beta1, beta2, eps;
   int grad_stride;  // floats between the rotating gradient buffers
   int persistent;   // 1: all steps in one cooperative launch
-  uint64_t mma_ns;  // tensor-core kernel: bound on the wait for a product (0: always run out)
+  // tensor-core kernel: bounds on the wait for a product (0: always run out) and
+  // on a grid barrier's (0: a CTA that would wait gives up at once)
+  uint64_t mma_ns, barrier_ns;
 };
 
 // The tensor-core training kernel (pdds_mlp_train_tc.cu): its function, grid,
@@ -48,10 +53,11 @@ cudaError_t train_tc_launch_config(bool adam, int64_t npts, const void** fn, uns
 
 }  // namespace pdds
 
-// pdds_mlp_train_tc with a bound of the caller's on the kernel's waits for its
-// products.  Not part of pdds.h: it lets a test make them run out.
+// pdds_mlp_train_tc with bounds of the caller's on the kernel's waits for its
+// products and, in the one launch, on its barriers'.  Not part of pdds.h: it
+// lets a test make them run out.
 extern "C" pdds_status pdds_internal_mlp_train_tc(float* theta, const float* xy,
                                                   const float* target, int64_t npts,
                                                   int32_t steps, double lr,
                                                   double* loss_history_host, void* cuda_stream,
-                                                  uint64_t mma_ns);
+                                                  uint64_t mma_ns, uint64_t barrier_ns);

@@ -536,7 +536,7 @@ namespace {
 pdds_status train_impl(int engine, const char* name, float* theta, const float* xy,
                        const float* target, int64_t npts, int32_t steps, double lr,
                        double* loss_history_host, void* cuda_stream,
-                       uint64_t mma_ns = kTrainWaitNs) {
+                       uint64_t mma_ns = kTrainWaitNs, uint64_t barrier_ns = kTrainWaitNs) {
   if (!theta || !xy || !target || npts < 1 || steps < 1 || !(lr > 0))
     return mlp_fail(PDDS_EINVAL,
                     std::string(name) + ": NULL pointer, npts < 1, steps < 1 or lr <= 0");
@@ -573,6 +573,7 @@ pdds_status train_impl(int engine, const char* name, float* theta, const float* 
   a.loss = reinterpret_cast<double*>(buf + sbytes + sizeof(TrainState));
   a.steps = steps;
   a.mma_ns = mma_ns;
+  a.barrier_ns = barrier_ns;
   a.lr = (float)lr;
   a.beta1 = 0.9f;
   a.beta2 = 0.999f;
@@ -588,13 +589,19 @@ pdds_status train_impl(int engine, const char* name, float* theta, const float* 
       void* args[] = {&pa};
       r = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(threads), args, smem, s);
       if (r == cudaSuccess) {
-        if (loss_history_host)
+        int finished = 0;
+        r = cudaMemcpyAsync(&finished, &a.st->finished, sizeof finished, cudaMemcpyDeviceToHost, s);
+        if (r == cudaSuccess && loss_history_host)
           r = cudaMemcpyAsync(loss_history_host, a.loss, steps * sizeof(double),
                               cudaMemcpyDeviceToHost, s);
         const cudaError_t done = cudaStreamSynchronize(s);
-        return r != cudaSuccess ? r : done;
+        if (r != cudaSuccess || done != cudaSuccess) return r != cudaSuccess ? r : done;
+        if (finished) return cudaSuccess;
+        // a barrier's wait ran out: from the start again, launch by launch
+        if ((r = cudaMemsetAsync(buf, 0, bytes, s)) != cudaSuccess) return r;
+      } else {
+        (void)cudaGetLastError();
       }
-      (void)cudaGetLastError();
     }
     // steps + 1 launches (gradients 0..steps-1, updates 1..steps) run as a
     // CUDA graph of 64 identical launches replayed on a private stream (the
@@ -665,9 +672,9 @@ extern "C" pdds_status pdds_internal_mlp_train_tc(float* theta, const float* xy,
                                                   const float* target, int64_t npts,
                                                   int32_t steps, double lr,
                                                   double* loss_history_host, void* cuda_stream,
-                                                  uint64_t mma_ns) {
+                                                  uint64_t mma_ns, uint64_t barrier_ns) {
   return train_impl(1, "mlp_train_tc", theta, xy, target, npts, steps, lr, loss_history_host,
-                    cuda_stream, mma_ns);
+                    cuda_stream, mma_ns, barrier_ns);
 }
 
 extern "C" pdds_status pdds_mlp_eval(const float* theta, const float* xy, int64_t npts, float* v,

@@ -30,7 +30,10 @@
 // with four-float reductions (a CTA's 4,417 reductions were 4,417 L2
 // transactions), 13.4 / 31.5 in one launch (more than one tile per SM: launch
 // by launch).  Waits on the tensor core are bounded (2 s); a wait
-// that runs out turns the step's loss into NaN.
+// that runs out turns the step's loss into NaN.  So are the waits at the
+// barrier (CTAs that other streams' work keeps from starting): the CTAs then
+// leave, theta, which only the last update writes, is as it was given, and the
+// caller starts again launch by launch, where no CTA waits for another.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -462,7 +465,10 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
     }
     break;
   } else {
-    if (!grad_pass) break;
+    if (!grad_pass) {
+      if (blockIdx.x == 0 && tid == 0) A.st->finished = 1;
+      break;
+    }
     p1 *= (double)A.beta1;
     p2 *= (double)A.beta2;
     // every CTA's gradient (and CTA 0's parameters) before anyone's next step
@@ -477,21 +483,18 @@ __global__ void __launch_bounds__(kThreads, 2) mlp_train_tc_kernel(const TrainAr
         unsigned seen;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&A.st->count) : "memory");
         if ((int)(seen - want) >= 0) break;
-        if ((spin & 255) == 0) {
+        if ((spin & 255) == 0 || A.barrier_ns == 0) {
           const uint64_t now = tc::now_ns();
           if (began == 0) began = now;
-          if (now - began > kTrainWaitNs) { met = false; break; }
+          if (now - began >= A.barrier_ns || __ldcg(&A.st->aborted) != 0) { met = false; break; }
         }
       }
       __threadfence();
+      if (!met) atomicExch(&A.st->aborted, 1);
       S.met = met ? 1 : 0;
     }
     __syncthreads();
-    if (!S.met) {  // a CTA is gone: every later loss is void
-      if (tid == 0)
-        for (int q = t + 1; q < A.steps; ++q) atomicAdd(A.loss + q, __longlong_as_double(0x7ff8000000000000ll));
-      break;
-    }
+    if (!S.met) break;
   }
   }
   tc::fence_before();
