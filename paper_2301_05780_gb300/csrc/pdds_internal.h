@@ -256,13 +256,17 @@ struct SolveJob {           // one problem of a batched solve
   double relres;            //   0 (maxit) or a negative breakdown code
   int converged;
 };
-// Solves every job (device pointers); synchronizes the stream.
+constexpr uint64_t kSolveWaitNs = 10000000000ull;
+// Solves every job (device pointers); synchronizes the stream.  wait_ns bounds
+// the wait at a barrier between the CTAs that share a problem; a problem whose
+// wait runs out is solved again on one CTA.
 cudaError_t bicgstab_batch(SolveJob* jobs, int count, double rtol, int32_t maxit, int* launches,
-                           cudaStream_t stream);
+                           cudaStream_t stream, uint64_t wait_ns = kSolveWaitNs);
 cudaError_t bicgstab_device(const int32_t* row_ptr, const int32_t* col, const double* val,
                             const double* b, double* x, int64_t n, int64_t nnz, double* work,
                             SolveScalars* sc, double rtol, int32_t maxit, int32_t* iters,
-                            double* relres, int* converged, int* launches, cudaStream_t stream);
+                            double* relres, int* converged, int* launches, cudaStream_t stream,
+                            uint64_t wait_ns = kSolveWaitNs);
 size_t bicgstab_work_doubles(int64_t n);
 void set_global_error(const std::string& msg);  // text of pdds_last_error(NULL)
 size_t bicgstab_scalars_bytes();
@@ -275,3 +279,9 @@ inline const char* bicgstab_stop_reason(int converged) {
 }
 
 }  // namespace pdds
+
+// pdds_solve_noalloc with a bound of the caller's on the barriers' waits.  Not
+// part of pdds.h: it lets a test make them run out.
+extern "C" pdds_status pdds_internal_solve_noalloc(const pdds_csr* G, const double* b, double* u,
+                                                   double rtol, int32_t maxit, int32_t* iters,
+                                                   void* cuda_stream, uint64_t wait_ns);

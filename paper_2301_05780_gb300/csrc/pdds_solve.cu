@@ -20,6 +20,9 @@
 // it arrives, and every CTA adds all of them in the same order after it, so
 // that all CTAs see the same bits, decide alike, and a solve repeats exactly.
 // Several problems share a launch, each on its own CTAs with its own barrier.
+// A barrier's wait is bounded (CTAs that other streams' work keeps from
+// starting); a problem whose wait has run out is solved again on one CTA,
+// which waits for no other.
 // Measured on one GB300 against six launches per iteration (one warp per row,
 // host read every eight iterations): 68 us per iteration instead of 200 on
 // 113,665 unknowns / 8.3e6 nonzeros (27 us of FP64 FMAs), 44 instead of 75 on
@@ -65,7 +68,7 @@ struct SolveDesc {
   SolveScalars* sc;   // up to the partial sums zeroed before the launch
   int64_t n;
   double rtol;
-  uint64_t wait_ns;   // bound on a barrier's wait
+  uint64_t wait_ns;   // bound on a barrier's wait (0: a CTA that would wait gives up at once)
   int32_t maxit, cta0, ctas, lanes;  // lanes of a warp that share a row
 };
 
@@ -99,11 +102,11 @@ struct Team {
       unsigned seen;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&sc->arrived) : "memory");
       if ((int)(seen - target) >= 0) break;
-      if ((spin & 255) == 255) {
+      if ((spin & 255) == 255 || wait_ns == 0) {
         uint64_t t;
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
         if (t0 == 0) t0 = t;
-        if (t - t0 > wait_ns) return false;
+        if (t - t0 >= wait_ns || __ldcg(&sc->timeout) != 0) return false;
       }
     }
     __threadfence();
@@ -316,24 +319,33 @@ __global__ void __launch_bounds__(kThreads, 1) k_bicgstab(const __grid_constant_
 size_t bicgstab_work_doubles(int64_t n) { return (size_t)6 * (size_t)n; }
 size_t bicgstab_scalars_bytes() { return sizeof(SolveScalars); }
 
-cudaError_t bicgstab_batch(SolveJob* jobs, int count, double rtol, int32_t maxit, int* launches,
-                           cudaStream_t st) {
-  int dev = 0, sms = 0;
+namespace {
+
+// One launch (per kInline problems) that solves jobs[which[0 .. count)] on at
+// most `most` CTAs, or on more if each problem gets just one; outcomes to
+// heads[which[..]] once the stream has been synchronized with.  `again`: after
+// a run of the same jobs, whose b may have been overwritten (u may be b's own
+// memory) and is taken from where that run kept it.
+struct SolveHead { double relres; int32_t converged, breakdown, iters, timeout; };
+
+cudaError_t launch_solves(const SolveJob* jobs, const std::vector<int>& which, int most, bool again,
+                          double rtol, int32_t maxit, uint64_t wait_ns, SolveHead* heads,
+                          int* launches, cudaStream_t st) {
   cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if (launches) *launches = 0;
+  const int count = (int)which.size();
   for (int base = 0; base < count; base += kInline) {
     SolveParams P{};
     P.count = std::min(kInline, count - base);
     int64_t total = 0;
-    for (int i = 0; i < P.count; ++i) total += std::max<int64_t>(jobs[base + i].nnz, 1);
-    for (int limit = sms;; limit /= 2) {
+    for (int i = 0; i < P.count; ++i) total += std::max<int64_t>(jobs[which[base + i]].nnz, 1);
+    for (int limit = most;; limit /= 2) {
       int ctas = 0;
       for (int i = 0; i < P.count; ++i) {
-        const SolveJob& J = jobs[base + i];
+        const SolveJob& J = jobs[which[base + i]];
         SolveDesc& D = P.inl[i];
-        D = SolveDesc{J.rp, J.ci, J.val, J.b, J.x, J.work, J.sc, J.n, rtol, 10000000000ull, maxit, 0, 0, 0};
+        // (the recurrence's shadow residual is b)
+        D = SolveDesc{J.rp, J.ci, J.val, again ? J.work + J.n : J.b, J.x, J.work, J.sc, J.n, rtol,
+                      wait_ns, maxit, 0, 0, 0};
         // One CTA up to 12 nonzeros a thread (its barriers stay inside the SM),
         // else one per two nonzeros a thread, at most its share of the SMs.
         const int64_t want = J.nnz <= 12 * kThreads ? 1 : (J.nnz + 2 * kThreads - 1) / (2 * kThreads);
@@ -366,18 +378,39 @@ cudaError_t bicgstab_batch(SolveJob* jobs, int count, double rtol, int32_t maxit
       break;
     }
     if (launches) *launches += 1;
+    for (int i = 0; i < P.count; ++i)
+      if ((e = cudaMemcpyAsync(&heads[which[base + i]], P.inl[i].sc, sizeof(SolveHead),
+                               cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+        return e;
   }
-  struct Head { double relres; int32_t converged, breakdown, iters, timeout; };
-  std::vector<Head> h(count);
+  return cudaStreamSynchronize(st);
+}
+
+}  // namespace
+
+cudaError_t bicgstab_batch(SolveJob* jobs, int count, double rtol, int32_t maxit, int* launches,
+                           cudaStream_t st, uint64_t wait_ns) {
+  int dev = 0, sms = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if (launches) *launches = 0;
+  std::vector<SolveHead> h(count);
+  std::vector<int> which(count);
+  for (int i = 0; i < count; ++i) which[i] = i;
+  if ((e = launch_solves(jobs, which, sms, false, rtol, maxit, wait_ns, h.data(), launches, st)) !=
+      cudaSuccess)
+    return e;
+  which.clear();
   for (int i = 0; i < count; ++i)
-    if ((e = cudaMemcpyAsync(&h[i], jobs[i].sc, sizeof(Head), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
-      return e;
-  if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+    if (h[i].timeout) which.push_back(i);
+  if (!which.empty() && (e = launch_solves(jobs, which, 1, true, rtol, maxit, wait_ns, h.data(),
+                                           launches, st)) != cudaSuccess)
+    return e;
   for (int i = 0; i < count; ++i) {
     jobs[i].iters = h[i].iters;
     jobs[i].relres = h[i].relres;
     jobs[i].converged = h[i].converged ? 1 : -h[i].breakdown;
-    if (h[i].timeout) return cudaErrorLaunchTimeout;
   }
   return cudaSuccess;
 }
@@ -385,9 +418,10 @@ cudaError_t bicgstab_batch(SolveJob* jobs, int count, double rtol, int32_t maxit
 cudaError_t bicgstab_device(const int32_t* rp, const int32_t* ci, const double* val,
                             const double* b, double* x, int64_t n, int64_t nnz, double* work,
                             SolveScalars* sc, double rtol, int32_t maxit, int32_t* iters,
-                            double* relres, int* converged, int* launches, cudaStream_t st) {
+                            double* relres, int* converged, int* launches, cudaStream_t st,
+                            uint64_t wait_ns) {
   SolveJob J{rp, ci, val, b, x, n, nnz, work, sc, 0, 0.0, 0};
-  const cudaError_t e = bicgstab_batch(&J, 1, rtol, maxit, launches, st);
+  const cudaError_t e = bicgstab_batch(&J, 1, rtol, maxit, launches, st, wait_ns);
   if (e != cudaSuccess) return e;
   if (iters) *iters = J.iters;
   if (relres) *relres = J.relres;
@@ -426,9 +460,9 @@ double* g_noalloc_ptr[kMaxDevices] = {nullptr};
 }  // namespace
 }  // namespace pdds
 
-extern "C" pdds_status pdds_solve_noalloc(const pdds_csr* G, const double* b, double* u,
-                                          double rtol, int32_t maxit, int32_t* iters,
-                                          void* cuda_stream) {
+extern "C" pdds_status pdds_internal_solve_noalloc(const pdds_csr* G, const double* b, double* u,
+                                                   double rtol, int32_t maxit, int32_t* iters,
+                                                   void* cuda_stream, uint64_t wait_ns) {
   using namespace pdds;
   if (!G || !b || !u || !G->row_ptr || !G->col || !G->val) {
     set_global_error("solve_noalloc: NULL matrix/vector");
@@ -481,7 +515,7 @@ extern "C" pdds_status pdds_solve_noalloc(const pdds_csr* G, const double* b, do
   // bicgstab_device zeroes the scalars and initialises every work vector it
   // reads, so the previous call's contents never leak into this one.
   e = bicgstab_device(G->row_ptr, G->col, G->val, b, u, G->n, G->nnz, scratch, sc, rtol, maxit, &it, &rel,
-                      &conv, &nl, (cudaStream_t)cuda_stream);
+                      &conv, &nl, (cudaStream_t)cuda_stream, wait_ns);
   if (e != cudaSuccess) {
     set_global_error(std::string("solve_noalloc: ") + cudaGetErrorString(e));
     return PDDS_ECUDA;
@@ -496,4 +530,10 @@ extern "C" pdds_status pdds_solve_noalloc(const pdds_csr* G, const double* b, do
     return PDDS_ENOCONV;
   }
   return PDDS_OK;
+}
+
+extern "C" pdds_status pdds_solve_noalloc(const pdds_csr* G, const double* b, double* u,
+                                          double rtol, int32_t maxit, int32_t* iters,
+                                          void* cuda_stream) {
+  return pdds_internal_solve_noalloc(G, b, u, rtol, maxit, iters, cuda_stream, pdds::kSolveWaitNs);
 }
