@@ -321,7 +321,7 @@ size_t bicgstab_scalars_bytes() { return sizeof(SolveScalars); }
 
 namespace {
 
-// One launch (per kInline problems) that solves jobs[which[0 .. count)] on at
+// One launch (for up to kInline problems) that solves jobs[which[0 .. count)] on at
 // most `most` CTAs, or on more if each problem gets just one; outcomes to
 // heads[which[..]] once the stream has been synchronized with.  `again`: after
 // a run of the same jobs, whose b may have been overwritten (u may be b's own
@@ -333,9 +333,17 @@ cudaError_t launch_solves(const SolveJob* jobs, const std::vector<int>& which, i
                           int* launches, cudaStream_t st) {
   cudaError_t e;
   const int count = (int)which.size();
-  for (int base = 0; base < count; base += kInline) {
+  for (int base = 0; base < count;) {
     SolveParams P{};
-    P.count = std::min(kInline, count - base);
+    // A context given twice has one scratch: its second solve goes into the
+    // next launch.
+    auto in_launch = [&](const SolveScalars* sc) {
+      for (int i = 0; i < P.count; ++i)
+        if (jobs[which[base + i]].sc == sc) return true;
+      return false;
+    };
+    while (P.count < kInline && base + P.count < count && !in_launch(jobs[which[base + P.count]].sc))
+      ++P.count;
     int64_t total = 0;
     for (int i = 0; i < P.count; ++i) total += std::max<int64_t>(jobs[which[base + i]].nnz, 1);
     for (int limit = most;; limit /= 2) {
@@ -382,6 +390,7 @@ cudaError_t launch_solves(const SolveJob* jobs, const std::vector<int>& which, i
       if ((e = cudaMemcpyAsync(&heads[which[base + i]], P.inl[i].sc, sizeof(SolveHead),
                                cudaMemcpyDeviceToHost, st)) != cudaSuccess)
         return e;
+    base += P.count;
   }
   return cudaStreamSynchronize(st);
 }
