@@ -744,7 +744,7 @@ __device__ __forceinline__ void step_calls(const PathConst& c, const KParams& P,
       if (!s.exited && s.n >= kmax) { s.exited = true; trunc = true; }
     }
   }
-  if (kPair && s.n + 2 * P.calls_per_check < kmax) {
+  if (kPair && below_cap(s.n, 2 * P.calls_per_check, kmax)) {
 #pragma unroll 1
     for (int call = P.calls_per_check; call > 0 && !s.exited; --call) {
       const uint4 r = kPre ? philox_step((uint32_t)(s.n >> 1), ph, P.round_keys)
@@ -1439,7 +1439,7 @@ __global__ void __launch_bounds__(CV == 1 ? 256 : 1024, CV == 1 ? 2 : 1)
         const int rounds = max(1, P.calls_per_check >> log2g);
         if (path_kernel_draws_ahead(COEF, CV, RECORD, EXT) && log2g > 0 && todo != 0 &&
             __all_sync(kFull, !((todo >> lane) & 1) ||
-                                  (!(n & 1) && n + ((2 * rounds) << log2g) < kmax))) {
+                                  (!(n & 1) && below_cap(n, (2 * rounds) << log2g, kmax)))) {
           if (kAngles && P.trig_direct) coop_calls<COEF, CV, EXT, kAngles>(c, P, todo, log2g, rounds, s);
           else coop_calls<COEF, CV, EXT, false>(c, P, todo, log2g, rounds, s);
         } else if (alive && !exited) {

@@ -196,6 +196,9 @@ __host__ __device__ inline int64_t auto_unit_paths(int64_t paths, const UnitRule
 }
 // Unit and record prefixes of per-knot budgets; unit_paths 0: auto_unit_paths
 // of `share` times the knots' paths (share: problems of the launch).
+// A path of n < kmax steps stays below its step cap for `more` steps (the cap
+// may be 2^31 - 1, so the sum n + more may not fit).
+__host__ __device__ inline bool below_cap(int n, int more, int kmax) { return more < kmax - n; }
 // Budgets outside [0, 2^31) count as zero paths and set *err = PDDS_EINVAL.
 cudaError_t launch_unit_prefix(const int64_t* n_per_knot, int64_t n, int64_t unit_paths,
                                int64_t share, const UnitRule& rule, int64_t* knot_unit_prefix,
