@@ -505,6 +505,18 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
   }
   // tcgen05 kernel: 96 TMEM columns per CTA, 512 per SM
   if (L.cv == 3) per_sm = std::min(per_sm, 512 / 96);
+  // The residents of a larger ring, none where a CTA cannot have that much (the
+  // limit counts the kernel's static shared memory too).
+  auto resident = [&](int block, size_t smem, int* ctas) {
+    *ctas = 0;
+    const cudaError_t e = pdds::allow_path_kernel_smem(coef_id, rec, L.cv, ext, smem);
+    if (e == cudaErrorInvalidValue) {
+      (void)cudaGetLastError();
+      return cudaSuccess;
+    }
+    return e != cudaSuccess ? e
+                            : pdds::path_kernel_occupancy(coef_id, rec, L.cv, ext, block, smem, ctas);
+  };
   // A unit's stage is free again only when its last path has left, so with two
   // stages the lanes run dry where units are short (per-knot budgets, wide
   // stencils, 128 lanes of the warpgroup kernel on 11-step paths).  More of
@@ -519,8 +531,7 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
     const int64_t ctas_all = (int64_t)c->num_sms * per_sm;
     if (units < r * ctas_all || smem * per_sm > (size_t)(L.cv == 2 ? 160 : 227) * 1024) continue;
     int ctas = 0;
-    CK(c, pdds::allow_path_kernel_smem(coef_id, rec, L.cv, ext, smem));
-    CK(c, pdds::path_kernel_occupancy(coef_id, rec, L.cv, ext, L.block, smem, &ctas));
+    CK(c, resident(L.block, smem, &ctas));
     if (ctas >= per_sm) {
       L.stages = r;
       L.smem = smem;
@@ -536,10 +547,7 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
     const int block = 384;
     const size_t smem = 3 * sbytes + net;
     int ctas = 0;
-    if (2 * smem <= 227 * 1024) {
-      CK(c, pdds::allow_path_kernel_smem(coef_id, rec, L.cv, ext, smem));
-      CK(c, pdds::path_kernel_occupancy(coef_id, rec, L.cv, ext, block, smem, &ctas));
-    }
+    if (2 * smem <= 227 * 1024) CK(c, resident(block, smem, &ctas));
     if (ctas == 2 && units >= 3 * 2 * (int64_t)c->num_sms) {
       L.block = block;
       L.stages = 3;
