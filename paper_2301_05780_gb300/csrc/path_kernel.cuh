@@ -720,6 +720,42 @@ __device__ __forceinline__ void step_selects(const PathConst& c, const KParams& 
     if (!s.exited && s.n >= kmax) { s.exited = true; trunc = true; }
   }
 }
+// The extended kernels of the tabulated set with the tabulated control variate:
+// step by step (below) and in scalars, one half of a call after the other, so
+// that the two lookups of a step overlap with the next half's arithmetic (GM
+// exits, 843 paths of 74 steps at 10,504 knots 8.25 -> 8.05 ms).
+template <int CV, bool DIRECT, bool MIXED>
+__device__ __forceinline__ void step_halves(const PathConst& c, const KParams& P, int kmax,
+                                            PathState& s, bool& trunc) {
+  constexpr int COEF = PDDS_COEF_TABLE;
+#pragma unroll 1
+  for (int call = P.calls_per_check; call > 0 && !s.exited; --call) {
+    const uint4 r = philox4x32_10(make_uint4((uint32_t)(s.n >> 1), c.p, c.kk, c.tagw), P.round_keys);
+    float z[4];
+    box_muller(r.x, r.y, z[0], z[1]);
+    box_muller(r.z, r.w, z[2], z[3]);
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      if (!s.exited && (!MIXED || half >= (s.n & 1))) {
+        float sg, ddx, ddy, cc, f;
+        coeffs<COEF>(*c.H, c.tile, c.tile, c.xk + s.X, c.yk + s.Y, s.X, s.Y, DIRECT, sg, ddx, ddy, cc, f);
+        const float Yw = ex2_approx(s.S);
+        s.Z = fmaf(-f * Yw, c.h, s.Z);
+        s.S = fmaf(cc, c.hl2, s.S);
+        const float ssh = sg * c.sqh;
+        float gx, gy;
+        cv_table_grad<true>(P.prob0, c.xk + s.X, c.yk + s.Y, gx, gy);
+        s.XI = fmaf(-Yw * ssh, fmaf(gx, z[2 * half], gy * z[2 * half + 1]), s.XI);
+        s.X = fmaf(ssh, z[2 * half], s.X);
+        s.Y = fmaf(ssh, z[2 * half + 1], s.Y);
+        ++s.n;
+        s.exited = left_patch<COEF, true>(*c.H, c.tile, c.xk, c.yk, s.X, s.Y, c.bx0, c.bx1, c.by0, c.by1,
+                                          c.gmc, DIRECT);
+        if (!s.exited && s.n >= kmax) { s.exited = true; trunc = true; }
+      }
+    }
+  }
+}
 template <int COEF, int CV, bool EXT, bool DIRECT, bool MIXED>
 __device__ __forceinline__ void step_calls(const PathConst& c, const KParams& P, const PhiloxPath& ph,
                                            int kmax, PathState& s, bool& trunc) {
@@ -729,6 +765,10 @@ __device__ __forceinline__ void step_calls(const PathConst& c, const KParams& P,
   constexpr bool kPair = !(EXT && COEF == PDDS_COEF_TABLE);
   if constexpr (uses_selects<COEF, CV, EXT>()) {
     step_selects<COEF, CV, DIRECT>(c, P, kmax, s, trunc);
+    return;
+  }
+  if constexpr (EXT && CV == 2 && COEF == PDDS_COEF_TABLE) {
+    step_halves<CV, DIRECT, MIXED>(c, P, kmax, s, trunc);
     return;
   }
   if constexpr (MIXED && kPair) {
