@@ -541,9 +541,12 @@ pdds_status plan_launch(pdds_ctx* c, int coef_id, bool rec, bool ext, int nprob,
   // Coefficient tiles that leave room for two stages only: fewer, larger CTAs
   // of three stages keep as many warps and wait less for a unit's last paths,
   // once units are long enough to be worth sharing (1,000 paths per knot 31.25 ->
-  // 30.05 ms, 2,000 4.34 -> 4.24; 300: 8.54 -> 8.74, so not below 512).
+  // 30.05 ms, 2,000 4.34 -> 4.24; 300: 8.54 -> 8.74, so not below 512), and where
+  // exits are rare enough that twelve warps can share a unit's FP64 sum of b (GM
+  // exits, 843 paths at 5,681 knots: 9 steps 1.44 -> 1.88 ms, 24 steps 1.97 -> 1.88;
+  // the naive exit sums across the warp first).
   if (coef_id == PDDS_COEF_TABLE && L.stages == 2 && L.cv != 1 && c->auto_block &&
-      c->ctas_per_sm <= 0 && per_knot >= 512) {
+      c->ctas_per_sm <= 0 && per_knot >= 512 && (!ext || mean_steps_estimate(c, dt) >= 20.0)) {
     const int block = 384;
     const size_t smem = 3 * sbytes + net;
     int ctas = 0;
