@@ -159,7 +159,7 @@ pdds_status pdds_set_step_cap(pdds_ctx* ctx, int64_t k_max);
  * Zeros keep the current value.  pdds_autotune picks them by measurement.  A
  * field that neither has set is the library's choice, launch by launch, from
  * the problem's paths, steps per path and shared memory; pdds_get_launch then
- * reports 256 / 0 / 4096 / 4. */
+ * reports the starting values 256 / 0 / 4096 / 4, which no launch need have. */
 pdds_status pdds_set_launch(pdds_ctx* ctx, int32_t block, int32_t ctas_per_sm,
                             int32_t unit_paths, int32_t exit_batch);
 pdds_status pdds_get_launch(const pdds_ctx* ctx, int32_t* block, int32_t* ctas_per_sm,
@@ -324,8 +324,11 @@ pdds_status pdds_assemble_batch(pdds_ctx* const* ctxs, int32_t count,
                                 void* cuda_stream);
 
 /* FP64 BiCGSTAB for G u = b (Eq. 23), all on the device; u (device double[n])
- * is overwritten (initial guess 0).  One cooperative kernel launch; synchronizes the
- * stream to read the outcome.  Returns ENOCONV if ||b - G u|| > rtol ||b||
+ * is overwritten (initial guess 0).  One kernel launch (cooperative but for systems
+ * small enough for one CTA); synchronizes the stream to read the outcome.  The CTAs of
+ * a system wait for one another at most 10 s at a time (other work on the device can
+ * keep some of them from starting); a system whose wait runs out is solved again, on
+ * one CTA, in a second launch.  Returns ENOCONV if ||b - G u|| > rtol ||b||
  * after maxit iterations; *iters (nullable) gets the iteration count. */
 pdds_status pdds_solve(pdds_ctx* ctx, const pdds_csr* G, const double* b, double* u,
                        double rtol, int32_t maxit, int32_t* iters, void* cuda_stream);
@@ -348,9 +351,10 @@ pdds_status pdds_mlp_loss_grad(const float* theta, const float* xy, const float*
 
 /* `steps` full-batch Adam steps (beta1 0.9, beta2 0.999, eps 1e-8, rate lr)
  * on the loss above; theta (DEVICE) is updated in place; loss_history_host
- * (nullable) receives the loss before each step.  Allocates and frees its own
- * scratch (gradient, Adam moments, step state, loss history) and a private
- * stream on which the steps run as a replayed CUDA graph, ordered after the
+ * (nullable) receives the loss before each step.  Its scratch (gradient, Adam
+ * moments, step state, loss history) is a static device array of 1 MB that the
+ * library's network calls share, or, when that is taken or too small, allocated and
+ * freed; it has a private stream on which the steps run as a replayed CUDA graph, ordered after the
  * work already queued on cuda_stream; synchronizes.  One kernel launch per
  * step: 64-point tiles on at most two CTAs per SM, FP32 throughout, the
  * CTA partial gradients added with FP32 atomics (the summation order, and so
@@ -370,9 +374,12 @@ pdds_status pdds_mlp_train(float* theta, const float* xy, const float* target, i
  * tcgen05.mma kind::f16 with BF16 operands and FP32 accumulation; the rest
  * is FP32.  The loss and the gradient carry the BF16 rounding of the
  * products' operands (within 1e-2 of the FP64 loss and gradient norm).
- * Arguments, the Adam step, scratch, graph replay and synchronisation as for
- * pdds_mlp_loss_grad / pdds_mlp_train.  A bounded tensor-core wait (2 s) that
- * runs out makes that step's loss NaN (loss, loss_history_host).
+ * Arguments, the Adam step, scratch and synchronisation as for
+ * pdds_mlp_loss_grad / pdds_mlp_train; the steps of a fit are one cooperative
+ * launch on cuda_stream, or, where that cannot be (or a wait of its CTAs for one
+ * another runs out, after 2 s), replayed launch by launch as there.  A bounded
+ * tensor-core wait (2 s) that runs out makes that step's loss NaN (loss,
+ * loss_history_host).
  * Errors: EINVAL, ECUDA. */
 pdds_status pdds_mlp_loss_grad_tc(const float* theta, const float* xy, const float* target,
                                   int64_t npts, float* grad, double* loss, void* cuda_stream);
@@ -403,8 +410,8 @@ pdds_status pdds_boundary_samples(const pdds_ctx* ctx, int32_t n_per_side, float
  * Eq. 37's grad v) each as three TF32 products of the hi / lo split of both
  * operands (FP32-accurate), the rest FP32.  Used to tabulate grad v_theta for
  * the look-up-table control variate (Sec. 4.2).  theta, xy [npts][2], v
- * (nullable) [npts], grad_xy [npts][2]: DEVICE.  One CTA of two 128-thread
- * warpgroups per SM (~195 KB of shared memory, 256 TMEM columns).
+ * (nullable) [npts], grad_xy [npts][2]: DEVICE.  One CTA of four 128-thread
+ * warpgroups per SM (~195 KB of shared memory, all 512 TMEM columns).
  * Synchronizes the stream.
  * Errors: EINVAL, ECUDA, ETIMEOUT (a bounded tensor-core wait ran out). */
 pdds_status pdds_mlp_eval_tc(const float* theta, const float* xy, int64_t npts, float* v,

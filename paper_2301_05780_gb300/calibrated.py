@@ -85,10 +85,10 @@ def run(w: W.Workload, eps: float, n0: int, h0: float, n_job: int, n0p: int | No
     lattice (pdds_boundary_samples), where u is known exactly.
     train_engine: the fit's training kernel ("fp32" or "tc", fit_network).
     launch: (block, unit_paths, exit_batch) of the path kernels, or None for
-    the library's default (256, 4096, 4).  The default here was measured on
-    the paper's problem, one GB300, over 15 shapes: 152 ms per pipeline
-    against 173 ms with the library's default (budgets of ~1,300 paths per
-    knot fill units of 1024 and give each CTA's ring short units).
+    the library's own rule.  The default is a fixed shape under which the
+    paper's problem has been measured throughout; the rule does as well (sum of
+    the phases, one GB300, eight pipelines each after a first: 145-156 ms with the default,
+    145-155 with None, 150-161 with 256 / 4096 / 4).
     Returns the nodal solutions of Phases I and III, the calibration (h_i,
     N_i, gap, var, rho^2), per-phase wall times (CUDA-synchronized) and
     path-step counts."""

@@ -15,7 +15,8 @@
 //    exited (exit times are wildly uneven, so lanes never wait for a whole
 //    batch of paths);
 //  - work units are (problem, knot, path range) taken from one global atomic
-//    queue; each CTA keeps two or three units at a time in shared memory (knot
+//    queue; each CTA keeps two or three units at a time (the network kernel up to
+//    eight) in shared memory (knot
 //    data, FP64 slot accumulators, TMA-staged coefficient tiles) so warps move
 //    on to the next unit while the stragglers of the previous one finish;
 //  - the warp that completes the last path of a unit flushes its accumulators
@@ -679,10 +680,10 @@ __device__ __forceinline__ void step_pair(const PathConst& c, const KParams& P, 
 // 1.5e11, the paper's GM warm-up, until then one branch per step, 20.1 -> 18.9
 // ms at 4.4e9, its production run 46.9 -> 45.3 ms).
 // With the tabulated control variate on the naive exit, the sets whose own step
-// leaves no registers for that form (the tabulated one and E1: 84 and 48 bytes
-// of spills against 0 and 12) keep the selects and compares (step_selects):
-// E1 at 60 steps a path 1.04 -> 0.96 ms per 1.6e6 paths, tabulated at 400 steps
-// 1.50 -> 1.44 ms per 5,800 paths, 15.6 -> 15.1 ms per 2.5e6.
+// leaves no registers for that form (E1 and the tabulated one) keep the selects
+// and compares (step_selects): 1.6e6 E1 paths of 60 steps 1.04 -> 0.96 ms (0.92
+// with the lookup in scalars), 14,000 tabulated paths of 300 steps 1.21 -> 1.02,
+// 2.5e6 of 400 steps 15.6 -> 15.1.
 // MIXED: a path of the mixed run resumes after its Gobet-Menozzi exit at any
 // step.  At an odd one it first takes the second half of its call by itself, so
 // that the lanes of a warp share the loop that follows (with the whole visit

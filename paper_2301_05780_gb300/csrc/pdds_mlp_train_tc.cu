@@ -28,8 +28,7 @@
 // launch per step.  One GB300, per step at 11,241 / 113,665 points: 21.3 / 58.1 us
 // with a launch per step and the gradient added one float at a time, 14.9 / 31.5
 // with four-float reductions (a CTA's 4,417 reductions were 4,417 L2
-// transactions), 13.4 / 31.5 in one launch (more than one tile per SM: launch
-// by launch).  Waits on the tensor core are bounded (2 s); a wait
+// transactions), 13.4 / 31.5 in one launch.  Waits on the tensor core are bounded (2 s); a wait
 // that runs out turns the step's loss into NaN.  So are the waits at the
 // barrier (CTAs that other streams' work keeps from starting): the CTAs then
 // leave, theta, which only the last update writes, is as it was given, and the
